@@ -1,7 +1,7 @@
 // sell_build.cu -- CRS -> SELL-C-sigma conversion on the GPU (Sec. 3.3-3.4).
 //
-// Pipeline (one stream, two host synchronisations):
-//   k_rowlen / k_colcheck   rowLen[i] = rpt[i+1] - rpt[i]; input validation;
+// Pipeline (one stream, three host synchronisations):
+//   k_rowlen                rowLen[i] = rpt[i+1] - rpt[i]; validation of rpt;
 //                           max row length and sum of squares (for Eq. "cv")
 //   -- sync 1: validation word, max row length --
 //   sorting scope sigma     sigma <= 1: identity (no permutation stored)
@@ -11,17 +11,21 @@
 //                           larger: stable LSD radix sort over the key
 //                             (window, maxlen - rowLen), 8-bit digits
 //   k_chunk_len             sorted row lengths srl[r], cl[c] = max (Eq. "max")
-//   scan                    cs = exclusive prefix sum of C * cl (cl[i] =
-//                           (cs[i+1]-cs[i])/C)
-//   -- sync 2: stored size cs[Nc] --
-//   k_scatter               entry j of sorted row r = c*C + l -> cs[c] + j*C + l,
-//                           zero padding (value 0, column 0), value rounding
+//   k_chunk_reduce/apply    cs = exclusive prefix sum of C * cl (cl[i] =
+//                           (cs[i+1]-cs[i])/C), long chunks, their work units
+//   -- sync 2: stored size cs[Nc], long chunks, work units --
+//   k_long_lists            the long chunks' work lists
+//   k_scatter_tiled         entry j of sorted row r = c*C + l -> cs[c] + j*C + l,
+//   (k_scatter)             zero padding (value 0, column 0), value rounding;
+//                           validation of col
+//   -- sync 3: validation word --
 //
 // Every sort key is unique (it ends in the row's position), so any correct
 // sort gives the stable order: ties in length keep the original row order.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "sell_internal.cuh"
@@ -57,44 +61,62 @@ inline int grid_for(int64_t n, int threads, int64_t cap = 1 << 20) {
 }
 
 // ------------------------------------------------------------ row lengths
-__global__ void k_rowlen(const int64_t *__restrict__ rpt, int64_t N, int64_t nnz,
-                         int32_t *__restrict__ rl, BuildStats *st) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+// Four rows per thread and step, one set of atomics per block: with one set
+// per warp of a 2432-block grid, the 58,000 atomics on one cache line took
+// most of the kernel's 32 us at 2M rows (24 MB: 3.5 us at 6.8 TB/s).
+__global__ void __launch_bounds__(256) k_rowlen(const int64_t *__restrict__ rpt, int64_t N, int64_t nnz,
+                                                int32_t *__restrict__ rl, BuildStats *st) {
+    __shared__ unsigned int werr[8];
+    __shared__ int wmx[8];
+    __shared__ unsigned long long wsq[8];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned int err = 0;
     int mx = 0;
     unsigned long long sq = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += stride) {
-        int64_t a = rpt[i], b = rpt[i + 1];
-        int64_t len = b - a;
-        if (i == 0 && a != 0) err |= kErrRpt0;
-        if (i == N - 1 && b != nnz) err |= kErrRptEnd;
-        if (len < 0) { err |= kErrRptOrder; len = 0; }
-        if (len > 0x7FFFFFFF) { err |= kErrRowLong; len = 0; }
-        rl[i] = (int32_t)len;
-        mx = max(mx, (int)len);
-        sq += (unsigned long long)len * (unsigned long long)len;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < N; i0 += 4 * stride) {
+        int64_t a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            a[q] = i < N ? rpt[i] : 0;
+            b[q] = i < N ? rpt[i + 1] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            if (i >= N) break;
+            int64_t len = b[q] - a[q];
+            if (i == 0 && a[q] != 0) err |= kErrRpt0;
+            if (i == N - 1 && b[q] != nnz) err |= kErrRptEnd;
+            if (len < 0) { err |= kErrRptOrder; len = 0; }
+            if (len > 0x7FFFFFFF) { err |= kErrRowLong; len = 0; }
+            rl[i] = (int32_t)len;
+            mx = max(mx, (int)len);
+            sq += (unsigned long long)len * (unsigned long long)len;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         err |= __shfl_xor_sync(0xffffffffu, err, o);
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         sq += __shfl_xor_sync(0xffffffffu, sq, o);
     }
+    const int warp = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
+        werr[warp] = err;
+        wmx[warp] = mx;
+        wsq[warp] = sq;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
+            err |= werr[i];
+            mx = max(mx, wmx[i]);
+            sq += wsq[i];
+        }
         if (err) atomicOr(&st->err, err);
         atomicMax(&st->max_rl, mx);
         atomicAdd(&st->sumsq, sq);
     }
-}
-
-__global__ void k_colcheck(const int32_t *__restrict__ col, int64_t nnz, int64_t ncols,
-                           BuildStats *st) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    bool bad = false;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz; j += stride) {
-        int32_t c = col[j];
-        bad |= (c < 0) | ((int64_t)c >= ncols);
-    }
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrCol);
 }
 
 // ------------------------------------------------- window sort (small sigma)
@@ -119,43 +141,58 @@ __global__ void k_window_sort(const int32_t *__restrict__ rl, int64_t N, int64_t
         skey[i] = k;
     }
     __syncthreads();
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
+    // A window length that is a power of two needs no merges across windows:
+    // its last stage sorts every window upwards.  Steps with j <= 32 exchange
+    // keys inside the 64 that one warp handles, so only the wider ones need
+    // the whole block to wait (21 of the 78 steps of 4096 keys).
+    const int kmax = (W & (W - 1)) == 0 ? (int)W : P;
+    for (int k = 2; k <= kmax; k <<= 1) {
+        for (int lj = __ffs(k) - 2; lj >= 0; --lj) {
+            const int j = 1 << lj;
             for (int t = threadIdx.x; t < (P >> 1); t += blockDim.x) {
-                int lo = 2 * j * (t / j) + (t % j);
-                int hi = lo + j;
-                bool up = (lo & k) == 0;
-                unsigned long long a = skey[lo], b = skey[hi];
+                const int lo = ((t >> lj) << (lj + 1)) | (t & (j - 1));
+                const int hi = lo + j;
+                const bool up = k == kmax || (lo & k) == 0;
+                const unsigned long long a = skey[lo], b = skey[hi];
                 if ((a > b) == up) { skey[lo] = b; skey[hi] = a; }
             }
-            __syncthreads();
+            if (j > 32 || (j == 1 && k >= 64)) __syncthreads();  // the next step is wider than a warp's keys
+            else __syncwarp();
         }
     }
+    __syncthreads();
     for (int i = threadIdx.x; i < nrow; i += blockDim.x)
         perm[base + i] = (int32_t)(base + (int64_t)(skey[i] & 0xFFFull));
 }
 
 // --------------------------------------------------- radix sort (large sigma)
-__global__ void k_radix_init(const int32_t *__restrict__ rl, int64_t N, int64_t sigma, int lbits,
-                             int max_rl, unsigned long long *__restrict__ key,
-                             int32_t *__restrict__ val) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += stride) {
-        unsigned long long w = (unsigned long long)(i / sigma);
-        key[i] = (w << lbits) | (unsigned long long)(max_rl - rl[i]);
-        val[i] = (int32_t)i;
+// The key of row i: (window, max_rl - rowLen).  The first pass computes it
+// from the row lengths (and the row number is the value), so no pass over
+// memory writes the initial pairs; KT is 32 bits where the key fits, which
+// halves what the later passes move.
+template <class KT, bool FIRST>
+__device__ __forceinline__ KT radix_key(const KT *__restrict__ key, const int32_t *__restrict__ rl, int64_t i,
+                                        uint32_t sigma, int lbits, int max_rl) {
+    if constexpr (FIRST) {
+        const KT len = (KT)(max_rl - rl[i]);
+        const uint32_t w = (uint32_t)i / sigma;
+        return w ? ((KT)w << lbits) | len : len;
+    } else {
+        return key[i];
     }
 }
 
-__global__ void k_radix_hist(const unsigned long long *__restrict__ key, int64_t N, int shift,
-                             int64_t ntiles, uint32_t *__restrict__ hist) {
+template <class KT, bool FIRST>
+__global__ void k_radix_hist(const KT *__restrict__ key, const int32_t *__restrict__ rl, int64_t N, uint32_t sigma,
+                             int lbits, int max_rl, int shift, int64_t ntiles, uint32_t *__restrict__ hist) {
     __shared__ uint32_t cnt[256];
     cnt[threadIdx.x] = 0;
     __syncthreads();
     const int64_t t0 = blockIdx.x * (int64_t)kRadixTile;
+#pragma unroll
     for (int r = 0; r < kRadixRounds; ++r) {
         int64_t i = t0 + r * kRadixThreads + threadIdx.x;
-        if (i < N) atomicAdd(&cnt[(key[i] >> shift) & 0xFF], 1u);
+        if (i < N) atomicAdd(&cnt[(radix_key<KT, FIRST>(key, rl, i, sigma, lbits, max_rl) >> shift) & 0xFF], 1u);
     }
     __syncthreads();
     hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
@@ -163,50 +200,64 @@ __global__ void k_radix_hist(const unsigned long long *__restrict__ key, int64_t
 
 // Stable scatter of one tile: items are taken in rounds of 256 (thread order
 // inside a round, rounds in order); an item's rank is the number of earlier
-// items of the tile with the same digit.
+// items of the tile with the same digit.  All rounds' items are loaded before
+// the first is ranked.
+template <class KT, bool FIRST>
 __global__ void __launch_bounds__(kRadixThreads)
-k_radix_scatter(const unsigned long long *__restrict__ kin, const int32_t *__restrict__ vin,
-                unsigned long long *__restrict__ kout, int32_t *__restrict__ vout, int64_t N,
-                int shift, int64_t ntiles, const int64_t *__restrict__ off) {
+k_radix_scatter(const KT *__restrict__ kin, const int32_t *__restrict__ vin, KT *__restrict__ kout,
+                int32_t *__restrict__ vout, const int32_t *__restrict__ rl, int64_t N, uint32_t sigma, int lbits,
+                int max_rl, int shift, int64_t ntiles, const int64_t *__restrict__ off) {
     __shared__ int64_t base[256];
-    __shared__ uint32_t running[256];
     __shared__ uint32_t wcount[kRadixThreads / 32][256];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    base[tid] = off[(int64_t)tid * ntiles + blockIdx.x];
-    running[tid] = 0;
     const int64_t t0 = blockIdx.x * (int64_t)kRadixTile;
+    KT k[kRadixRounds];
+    int32_t v[kRadixRounds];
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r) {
+        const int64_t i = t0 + r * kRadixThreads + tid;
+        k[r] = i < N ? radix_key<KT, FIRST>(kin, rl, i, sigma, lbits, max_rl) : (KT)0;
+        v[r] = FIRST ? (int32_t)i : (i < N ? vin[i] : 0);
+    }
+    base[tid] = off[(int64_t)tid * ntiles + blockIdx.x];
     const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
     for (int r = 0; r < kRadixRounds; ++r) {
         for (int w = 0; w < kRadixThreads / 32; ++w) wcount[w][tid] = 0;
         __syncthreads();
-        int64_t i = t0 + r * kRadixThreads + tid;
-        bool valid = i < N;
-        unsigned long long k = valid ? kin[i] : 0ull;
-        int32_t v = valid ? vin[i] : 0;
-        unsigned d = valid ? (unsigned)((k >> shift) & 0xFF) : 256u;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        unsigned rank = __popc(peers & lt);
+        const bool valid = t0 + r * kRadixThreads + tid < N;
+        const unsigned d = valid ? (unsigned)((k[r] >> shift) & 0xFF) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const unsigned rank = __popc(peers & lt);
         if (valid && rank == 0) wcount[warp][d] = __popc(peers);
         __syncthreads();
-        if (valid) {
-            uint32_t pre = 0;
-            for (int w = 0; w < warp; ++w) pre += wcount[w][d];
-            int64_t pos = base[d] + running[d] + pre + rank;
-            kout[pos] = k;
-            vout[pos] = v;
+        // column tid of the counts: exclusive prefix over the warps
+        uint32_t tot = 0;
+        for (int w = 0; w < kRadixThreads / 32; ++w) {
+            const uint32_t n = wcount[w][tid];
+            wcount[w][tid] = tot;
+            tot += n;
         }
         __syncthreads();
-        uint32_t tot = 0;
-        for (int w = 0; w < kRadixThreads / 32; ++w) tot += wcount[w][tid];
-        running[tid] += tot;
+        if (valid) {
+            const int64_t pos = base[d] + wcount[warp][d] + rank;
+            kout[pos] = k[r];
+            vout[pos] = v[r];
+        }
         __syncthreads();
+        base[tid] += tot;
     }
 }
 
 // -------------------------------------------------------------- prefix scan
-// Exclusive scan of mult * in[i] (int64 result, out has n + 1 entries with the
-// total in out[n]).  Three kernels: tile sums, scan of tile sums (recursive),
-// tile scan plus offset.
+// Exclusive scan of int64 sums: out has n + 1 entries with the total in
+// out[n].  Two kernels: sums of 4096-item tiles, then every tile scans its
+// items and adds the sum of the tiles before it, which its block adds up
+// itself -- one launch less than a scan of the tile sums in between (3 us of
+// a small build's every scan); only above kScanFlat tiles, where that sum
+// would cost more than it saves, the tile sums are scanned first.
+constexpr int64_t kScanFlat = 4096;
+
 __device__ __forceinline__ int64_t block_exclusive(int64_t v, int64_t *warp_tot, int64_t *total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t inc = v;
@@ -231,47 +282,62 @@ __device__ __forceinline__ int64_t block_exclusive(int64_t v, int64_t *warp_tot,
     return inc - v + warp_tot[warp];
 }
 
+// The sum of bsum[0..n) (tile sums before this block's tile), by the whole block.
+__device__ __forceinline__ int64_t tiles_before(const int64_t *__restrict__ bsum, int64_t n, int64_t *wt) {
+    int64_t s = 0;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += bsum[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) wt[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += wt[i];
+    __syncthreads();
+    return s;
+}
+
 template <class T>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_reduce(const T *__restrict__ in, int64_t mult, int64_t n, int64_t *__restrict__ bsum) {
+k_scan_reduce(const T *__restrict__ in, int64_t n, int64_t *__restrict__ bsum) {
     __shared__ int64_t wt[32];
     __shared__ int64_t tot;
     int64_t i0 = blockIdx.x * (int64_t)kScanTile + threadIdx.x * kScanItems;
     int64_t s = 0;
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q)
-        if (i0 + q < n) s += (int64_t)in[i0 + q] * mult;
+        if (i0 + q < n) s += (int64_t)in[i0 + q];
     block_exclusive(s, wt, &tot);
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
+// boff: scanned tile sums; bsum: plain tile sums (added up here); neither
+// with a single tile.
 template <class T>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_apply(const T *__restrict__ in, int64_t mult, int64_t n, const int64_t *__restrict__ boff,
-             int64_t *__restrict__ out) {
+k_scan_apply(const T *__restrict__ in, int64_t n, const int64_t *__restrict__ boff,
+             const int64_t *__restrict__ bsum, int64_t *__restrict__ out) {
     __shared__ int64_t wt[32];
     __shared__ int64_t tot;
+    const int64_t before = boff ? boff[blockIdx.x] : (bsum ? tiles_before(bsum, blockIdx.x, wt) : 0);
     int64_t i0 = blockIdx.x * (int64_t)kScanTile + threadIdx.x * kScanItems;
     int64_t v[kScanItems];
     int64_t s = 0;
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
-        v[q] = (i0 + q < n) ? (int64_t)in[i0 + q] * mult : 0;
+        v[q] = (i0 + q < n) ? (int64_t)in[i0 + q] : 0;
         s += v[q];
     }
-    int64_t ex = block_exclusive(s, wt, &tot) + (boff ? boff[blockIdx.x] : 0);
+    int64_t ex = block_exclusive(s, wt, &tot) + before;
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
         if (i0 + q < n) out[i0 + q] = ex;
         ex += v[q];
     }
     // the tile total (items past n are zero) completes the last tile
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = (boff ? boff[blockIdx.x] : 0) + tot;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + tot;
 }
 
 template <class T>
-sell_status scan_exclusive(const T *in, int64_t mult, int64_t n, int64_t *out, const Allocator &al,
-                           cudaStream_t s) {
+sell_status scan_exclusive(const T *in, int64_t n, int64_t *out, const Allocator &al, cudaStream_t s) {
     if (n == 0) {
         SELL_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(int64_t), s));
         return SELL_OK;
@@ -280,21 +346,112 @@ sell_status scan_exclusive(const T *in, int64_t mult, int64_t n, int64_t *out, c
     DevBuf bsum, boff;
     if (nb > 1) {
         SELL_TRY(bsum.alloc(al, nb * sizeof(int64_t), s));
-        SELL_TRY(boff.alloc(al, (nb + 1) * sizeof(int64_t), s));
-        k_scan_reduce<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, mult, n, bsum.as<int64_t>());
+        k_scan_reduce<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum.as<int64_t>());
         SELL_CUDA_TRY(cudaGetLastError());
-        SELL_TRY(scan_exclusive<int64_t>(bsum.as<int64_t>(), 1, nb, boff.as<int64_t>(), al, s));
+        if (nb > kScanFlat) {
+            SELL_TRY(boff.alloc(al, (nb + 1) * sizeof(int64_t), s));
+            SELL_TRY(scan_exclusive<int64_t>(bsum.as<int64_t>(), nb, boff.as<int64_t>(), al, s));
+        }
     }
-    k_scan_apply<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, mult, n,
-                                                          nb > 1 ? boff.as<int64_t>() : nullptr, out);
+    k_scan_apply<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, boff.as<int64_t>(), bsum.as<int64_t>(), out);
     SELL_CUDA_TRY(cudaGetLastError());
     return SELL_OK;
 }
 
+// The three sums over the chunks in one scan: chunk offsets (C * cl), long
+// chunks (cl > kSeg) and their segments (ceil(cl / kSeg) each).
+struct ChunkSums {
+    int64_t stored, nlong, nunits;
+    __device__ __forceinline__ ChunkSums &operator+=(const ChunkSums &o) {
+        stored += o.stored;
+        nlong += o.nlong;
+        nunits += o.nunits;
+        return *this;
+    }
+};
+__device__ __forceinline__ ChunkSums sums_of(int32_t cl, int C) {
+    const bool lg = cl > kSeg;
+    return {(int64_t)C * cl, lg ? 1 : 0, lg ? (cl - 1) / kSeg + 1 : 0};  // no overflow near 2^31
+}
+__device__ __forceinline__ ChunkSums shfl_up(const ChunkSums &v, int o) {
+    return {__shfl_up_sync(0xffffffffu, v.stored, o), __shfl_up_sync(0xffffffffu, v.nlong, o),
+            __shfl_up_sync(0xffffffffu, v.nunits, o)};
+}
+// Inclusive scan over the block (1024 threads); *tot = the block's total.
+__device__ __forceinline__ ChunkSums block_inclusive(ChunkSums v, ChunkSums *wt) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const ChunkSums u = shfl_up(v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) wt[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        ChunkSums t = wt[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const ChunkSums u = shfl_up(t, o);
+            if (lane >= o) t += u;
+        }
+        __syncwarp();
+        wt[lane] = t;
+    }
+    __syncthreads();
+    if (warp > 0) v += wt[warp - 1];
+    return v;
+}
+
+// Sums of tiles of `per` chunks (a multiple of 1024), one tile per block.
+__global__ void __launch_bounds__(kScanThreads)
+k_chunk_reduce(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, ChunkSums *__restrict__ tile) {
+    __shared__ ChunkSums wt[32];
+    const int64_t c0 = blockIdx.x * per, c1 = min(Nc, c0 + per);
+    ChunkSums v = {0, 0, 0};
+    for (int64_t c = c0 + threadIdx.x; c < c1; c += kScanThreads) v += sums_of(cl[c], C);
+    v = block_inclusive(v, wt);
+    if (threadIdx.x == kScanThreads - 1) tile[blockIdx.x] = v;
+}
+
+// cs, and for the long chunks their index and first unit in lpos/ubase; the
+// totals go to cs[Nc] and *total.  tile: the tile sums.
+__global__ void __launch_bounds__(kScanThreads)
+k_chunk_apply(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, const ChunkSums *__restrict__ tile,
+              int64_t *__restrict__ cs, int64_t *__restrict__ lpos, int64_t *__restrict__ ubase,
+              ChunkSums *__restrict__ total) {
+    __shared__ ChunkSums wt[32];
+    __shared__ ChunkSums before;
+    ChunkSums s = {0, 0, 0};
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) s += tile[i];
+    s = block_inclusive(s, wt);
+    if (threadIdx.x == kScanThreads - 1) before = s;
+    __syncthreads();
+    const int64_t c1 = min(Nc, (blockIdx.x + 1) * per);
+    for (int64_t c0 = blockIdx.x * per; c0 < c1; c0 += kScanThreads) {
+        const int64_t c = c0 + threadIdx.x;
+        const ChunkSums own = sums_of(c < c1 ? cl[c] : 0, C);
+        ChunkSums v = block_inclusive(own, wt);
+        v += before;
+        if (c < c1) {
+            cs[c] = v.stored - own.stored;
+            lpos[c] = v.nlong - own.nlong;
+            ubase[c] = v.nunits - own.nunits;
+            if (c == Nc - 1) {
+                cs[Nc] = v.stored;
+                *total = v;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == kScanThreads - 1) before = v;
+        __syncthreads();
+    }
+}
+
 // ------------------------------------------------------------- chunk lengths
+// srl, cl, and src[r] = where sorted row r's entries begin in the CRS arrays:
+// the scatter then waits for one load instead of a chain of three (length,
+// perm, rpt) before a row's entries.
 __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__restrict__ perm,
-                            int64_t N, int64_t Np, int C, int32_t *__restrict__ srl,
-                            int32_t *__restrict__ cl, int32_t *__restrict__ inv) {
+                            const int64_t *__restrict__ rpt, int64_t N, int64_t Np, int C, int32_t *__restrict__ srl,
+                            int64_t *__restrict__ src, int32_t *__restrict__ cl, int32_t *__restrict__ inv) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool warp_chunks = (C % 32) == 0;
     // the loop trip count is uniform across a warp because Np is a multiple of
@@ -308,7 +465,10 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
             len = rl[old];
             if (inv) inv[old] = (int32_t)r;
         }
-        if (live) srl[r] = len;
+        if (live) {
+            srl[r] = len;
+            if (r < N) src[r] = rpt[perm ? perm[r] : r];
+        }
         if (warp_chunks) {
             int32_t m = len;
             for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -320,56 +480,38 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
 }
 
 // ---------------------------------------------------------- long-row chunks
-__global__ void k_long_flags(const int32_t *__restrict__ cl, int64_t Nc, int32_t *__restrict__ flag) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < Nc; c += stride)
-        flag[c] = cl[c] > kSeg ? 1 : 0;
-}
-
-__global__ void k_long_compact(const int32_t *__restrict__ cl, const int64_t *__restrict__ pos, int64_t Nc,
-                               int32_t *__restrict__ lchunk) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < Nc; c += stride)
-        if (cl[c] > kSeg) lchunk[pos[c]] = (int32_t)c;
-}
-
-// Long-row work units: chunk lc has ceil(cl / kSeg) segments; the units are
-// numbered chunk by chunk (ubase = exclusive scan of the segment counts).
-__global__ void k_long_nseg(const int32_t *__restrict__ cl, const int32_t *__restrict__ lchunk,
-                            int64_t nlong, int32_t *__restrict__ nseg) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlong; i += stride)
-        nseg[i] = (cl[lchunk[i]] - 1) / kSeg + 1;  // cl > kSeg for a long chunk
-}
-
-__global__ void k_long_units(const int32_t *__restrict__ nseg, const int64_t *__restrict__ ubase,
-                             int64_t nlong, int2 *__restrict__ lunit) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlong; i += stride)
-        for (int32_t sg = 0; sg < nseg[i]; ++sg) lunit[ubase[i] + sg] = make_int2((int)i, sg);
-}
-
-// Long rows of each long chunk: lrow[i*C + k] = the lane of its k-th row
-// longer than kSeg (lane order), lmeta[i] = {m rows, mode, units of the
-// chunk, 0}.  Mode 0: unit thread t takes lane t (its row's segment); mode 1,
-// for chunks whose long rows are few (8 m <= C): the chunk's unit threads
-// take consecutive segments of one long row after another, so a warp runs 32
-// segments of a long row instead of one segment of each of 32 mostly short
-// rows.  Either way each segment is the same chain and lands in the same
-// partial slot (unit of the segment, lane of the row), so the results do not
-// depend on the mode.
-__global__ void k_long_rows(const int32_t *__restrict__ srl, int64_t N, int C, const int32_t *__restrict__ lchunk,
-                            const int32_t *__restrict__ nseg, int64_t nlong, int32_t *__restrict__ lrow,
-                            int4 *__restrict__ lmeta) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlong; i += stride) {
-        const int64_t c = lchunk[i];
-        int m = 0;
-        for (int l = 0; l < C; ++l) {
-            const int64_t r = c * C + l;
-            if (r < N && srl[r] > kSeg) lrow[i * C + m++] = l;
-        }
-        lmeta[i] = make_int4(m, 8 * m <= C ? 1 : 0, nseg[i], 0);
+// The long chunks (cl > kSeg), one warp per chunk: lchunk[i] = the i-th
+// long chunk; its ceil(cl / kSeg) work units are lunit[ubase + s] = {i, s};
+// lrow[i*C + k] = the lane of its k-th row longer than kSeg (lane order),
+// lmeta[i] = {m rows, mode, units of the chunk, 0}.  Mode 0: unit thread t
+// takes lane t (its row's segment); mode 1, for chunks whose long rows are
+// few (8 m <= C): the chunk's unit threads take consecutive segments of one
+// long row after another, so a warp runs 32 segments of a long row instead of
+// one segment of each of 32 mostly short rows.  Either way each segment is
+// the same chain and lands in the same partial slot (unit of the segment,
+// lane of the row), so the results do not depend on the mode.
+__global__ void __launch_bounds__(256)
+k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, const int64_t *__restrict__ lpos,
+             const int64_t *__restrict__ ubase, int64_t Nc, int64_t N, int C, int32_t *__restrict__ lchunk,
+             int2 *__restrict__ lunit, int32_t *__restrict__ lrow, int4 *__restrict__ lmeta) {
+    const int lane = threadIdx.x & 31;
+    const int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int32_t width = c < Nc ? cl[c] : 0;
+    if (width <= kSeg) return;
+    const int64_t i = lpos[c], u = ubase[c];
+    const int nseg = (width - 1) / kSeg + 1;
+    for (int sg = lane; sg < nseg; sg += 32) lunit[u + sg] = make_int2((int)i, sg);
+    int m = 0;
+    for (int l0 = 0; l0 < C; l0 += 32) {
+        const int64_t r = c * C + l0 + lane;
+        const bool lg = l0 + lane < C && r < N && srl[r] > kSeg;
+        const unsigned hit = __ballot_sync(0xffffffffu, lg);
+        if (lg) lrow[i * C + m + __popc(hit & ((1u << lane) - 1u))] = l0 + lane;
+        m += __popc(hit);
+    }
+    if (lane == 0) {
+        lchunk[i] = (int32_t)c;
+        lmeta[i] = make_int4(m, 8 * m <= C ? 1 : 0, nseg, 0);
     }
 }
 
@@ -437,64 +579,260 @@ template <> __device__ __forceinline__ __nv_bfloat16 zero_of<__nv_bfloat16>() {
 }
 
 // One thread per sorted row; the C threads of a chunk write one stored column
-// (C consecutive elements) per step j, so stores are coalesced for C >= 32.
+// (C consecutive elements) per step j.  Chunk heights that are not a multiple
+// of 32 only: there a warp's rows span several chunks.
 template <class TI, class TO>
-__global__ void k_scatter(const int64_t *__restrict__ rpt, const int32_t *__restrict__ col_in,
-                          const TI *__restrict__ val_in, const int32_t *__restrict__ perm,
-                          const int32_t *__restrict__ inv, const int32_t *__restrict__ srl,
+__global__ void k_scatter(const int64_t *__restrict__ src_of, const int32_t *__restrict__ col_in,
+                          const TI *__restrict__ val_in, const int32_t *__restrict__ inv, const int32_t *__restrict__ srl,
                           const int32_t *__restrict__ cl, const int64_t *__restrict__ cs, int64_t N,
-                          int64_t Np, int C, TO *__restrict__ val, int32_t *__restrict__ col) {
+                          int64_t Np, int C, int64_t ncols, TO *__restrict__ val, int32_t *__restrict__ col,
+                          BuildStats *st) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    bool bad = false;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < Np; r += stride) {
         int64_t c = r / C;
         int l = (int)(r - c * C);
         int32_t width = cl[c];
         int32_t len = srl[r];
         int64_t src = 0;
-        if (r < N && len > 0) src = rpt[perm ? perm[r] : r];
+        if (r < N) src = src_of[r];
         int64_t pos = cs[c] + l;
         for (int32_t j = 0; j < width; ++j, pos += C) {
             if (j < len) {
                 int32_t cidx = col_in[src + j];
+                const bool out = cidx < 0 || (int64_t)cidx >= ncols;
+                bad |= out;
                 val[pos] = cvt<TI, TO>(val_in[src + j]);
-                col[pos] = inv ? inv[cidx] : cidx;
+                col[pos] = inv && !out ? inv[cidx] : cidx;
             } else {
                 val[pos] = zero_of<TO>();
                 col[pos] = 0;
             }
         }
     }
+    if (bad) atomicOr(&st->err, kErrCol);
 }
 
-template <class TI>
-sell_status launch_scatter(const sell_csr &A, const int64_t *rpt, const int32_t *col_in,
-                           const void *val_in, const int32_t *perm, const int32_t *inv,
-                           const int32_t *srl, const int32_t *cl, const int64_t *cs, int64_t Np,
-                           int C, int store, void *val, int32_t *col, cudaStream_t s) {
-    int g = grid_for(Np, 256);
-    const TI *vi = static_cast<const TI *>(val_in);
-    switch (store) {
-        case SELL_F64:
-            k_scatter<TI, double><<<g, 256, 0, s>>>(rpt, col_in, vi, perm, inv, srl, cl, cs, A.nrows,
-                                                    Np, C, (double *)val, col);
-            break;
-        case SELL_F32:
-            k_scatter<TI, float><<<g, 256, 0, s>>>(rpt, col_in, vi, perm, inv, srl, cl, cs, A.nrows,
-                                                   Np, C, (float *)val, col);
-            break;
-        default:
-            k_scatter<TI, __nv_bfloat16><<<g, 256, 0, s>>>(rpt, col_in, vi, perm, inv, srl, cl, cs,
-                                                           A.nrows, Np, C, (__nv_bfloat16 *)val, col);
-            break;
+// Chunk heights of a multiple of 32: one warp per slice (32 consecutive sorted
+// rows) and kSeg stored columns, kTileCols of them at a time.  The warp reads
+// the entries row by row -- 16 consecutive entries of two rows per load (4 or
+// 8 of more rows where the rows are short), so a row's bytes are read once and
+// in whole sectors -- into a shared tile, and writes the tile column by column
+// (32 consecutive elements).  The first Np /
+// 32 warps take each slice's first kSeg columns, the others the long chunks'
+// further segments (lunit), so one very long row does not hold a single warp
+// for its whole length.
+// Bound: HBM (CRS read once, the format written once: 770 MB and 113 us at
+// 6.8 TB/s for 2M lognormal rows in binary64).  The thread-per-row form above
+// took 648 us there (two dependent uncoalesced loads in flight per thread),
+// this one 235 us: the rows' pieces begin and end inside sectors (1.46 times
+// the bytes move) and the warp waits for each batch of loads.  Loads in
+// flight: 8 per lane for 8-byte values (235 us; 4: 283 us), 4 for the others
+// (1M banded rows to binary32 80 us; 8: 94 us); a branch around each load
+// instead of a predicate cost up to 60 % more.
+constexpr int kTileCols = 16;
+
+// A read-only load under a predicate, zero otherwise, with no branch around
+// it: a batch of them is in flight together.
+__device__ __forceinline__ double ld_if(const double *p, bool on) {
+    double v;
+    asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.f64 %0, 0d0000000000000000;\n @q ld.global.nc.f64 %0, [%1];\n}"
+        : "=d"(v) : "l"(p), "r"((int)on));
+    return v;
+}
+__device__ __forceinline__ float ld_if(const float *p, bool on) {
+    float v;
+    asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.f32 %0, 0f00000000;\n @q ld.global.nc.f32 %0, [%1];\n}"
+        : "=f"(v) : "l"(p), "r"((int)on));
+    return v;
+}
+__device__ __forceinline__ int32_t ld_if(const int32_t *p, bool on) {
+    int32_t v;
+    asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.s32 %0, 0;\n @q ld.global.nc.s32 %0, [%1];\n}"
+        : "=r"(v) : "l"(p), "r"((int)on));
+    return v;
+}
+constexpr int kScatterWarps = 4;
+
+template <class TI, class TO>
+__global__ void __launch_bounds__(kScatterWarps * 32)
+k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ col_in,
+                const TI *__restrict__ val_in, const int32_t *__restrict__ inv, const int32_t *__restrict__ srl,
+                const int32_t *__restrict__ cl, const int64_t *__restrict__ cs, const int32_t *__restrict__ lchunk,
+                const int2 *__restrict__ lunit, int64_t nunits, int64_t N, int64_t nslices, int C, int64_t ncols,
+                TO *__restrict__ val, int32_t *__restrict__ col, BuildStats *st) {
+    // row pitches that keep the column-wise writes of a half-warp off each
+    // other's banks
+    __shared__ TO tval[kScatterWarps][kTileCols][sizeof(TO) == 8 ? 33 : 34];
+    __shared__ int32_t tcol[kScatterWarps][kTileCols][34];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t w = blockIdx.x * (int64_t)kScatterWarps + warp;
+    const uint32_t spc = (uint32_t)C / 32;  // slices per chunk
+    int64_t c;
+    uint32_t sl;
+    int seg = 0;
+    if (w < nslices) {
+        c = (uint32_t)w / spc;
+        sl = (uint32_t)w % spc;
+    } else {
+        const int64_t i = w - nslices;
+        if (i >= nunits * spc) return;
+        const int2 us = lunit[i / spc];
+        seg = us.y;
+        if (seg == 0) return;  // the slice's own warp has the first segment
+        sl = (uint32_t)(i % spc);
+        c = lchunk[us.x];
+    }
+    const int64_t slice = c * spc + sl, r = slice * 32 + lane;
+    const int64_t cs0 = cs[c];
+    const int j0 = seg * kSeg, j1 = min(cl[c], j0 + kSeg);
+    const int len = r < N ? srl[r] : 0;
+    const int64_t src = r < N ? src_of[r] : 0;
+    const int wmax = __reduce_max_sync(0xffffffffu, len);
+    bool bad = false;
+    auto mapped = [&](int32_t cidx) {
+        const bool out = cidx < 0 || (int64_t)cidx >= ncols;
+        bad |= out;
+        return inv && !out ? inv[cidx] : cidx;
+    };
+    auto load_tile = [&](auto lanes_log2, int jt) {
+        constexpr int LG = decltype(lanes_log2)::value;
+        constexpr int B = sizeof(TO) == 8 ? 8 : 4;  // loads in flight per lane and array, at most 1 << LG
+        constexpr int BB = B < (1 << LG) ? B : (1 << LG);
+        const int jj = lane & ((1 << LG) - 1);
+#pragma unroll 1
+        for (int it = 0; it < (1 << LG); it += BB) {
+            TI v[BB];
+            int32_t ci[BB];
+            bool in[BB];
+#pragma unroll
+            for (int b = 0; b < BB; ++b) {
+                const int l = ((it + b) << (5 - LG)) + (lane >> LG);
+                const int n = __shfl_sync(0xffffffffu, len, l);
+                const int64_t p = __shfl_sync(0xffffffffu, src, l) + jt + jj;
+                in[b] = jt + jj < n;
+                v[b] = ld_if(val_in + p, in[b]);
+                ci[b] = ld_if(col_in + p, in[b]);
+            }
+#pragma unroll
+            for (int b = 0; b < BB; ++b) {
+                const int l = ((it + b) << (5 - LG)) + (lane >> LG);
+                tval[warp][jj][l] = cvt<TI, TO>(v[b]);  // zero stays zero
+                tcol[warp][jj][l] = in[b] ? mapped(ci[b]) : 0;
+            }
+        }
+    };
+    for (int jt = j0; jt < j1; jt += kTileCols) {
+        if (jt < wmax) {
+            // 16 lanes per row, fewer where the rest of the rows is short
+            const int rest = wmax - jt;
+            if (rest > 8) load_tile(std::integral_constant<int, 4>(), jt);
+            else if (rest > 4) load_tile(std::integral_constant<int, 3>(), jt);
+            else load_tile(std::integral_constant<int, 2>(), jt);
+            __syncwarp();
+        }
+        const int nj = min(kTileCols, j1 - jt);
+        int64_t pos = cs0 + (int64_t)jt * C + sl * 32 + lane;
+        for (int q = 0; q < nj; ++q, pos += C) {
+            if (jt + q < wmax) {
+                val[pos] = tval[warp][q][lane];
+                col[pos] = tcol[warp][q][lane];
+            } else {  // columns that only other slices of the chunk reach
+                val[pos] = zero_of<TO>();
+                col[pos] = 0;
+            }
+        }
+        __syncwarp();
+    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&st->err, kErrCol);
+}
+
+// Arrays of the format under construction that the scatter reads or writes.
+struct ScatterArgs {
+    const int64_t *src;
+    const int32_t *col_in;
+    const void *val_in;
+    const int32_t *inv, *srl, *cl;
+    const int64_t *cs;
+    const int32_t *lchunk;
+    const int2 *lunit;
+    int64_t nunits, N, Np, ncols;
+    int C;
+    void *val;
+    int32_t *col;
+    BuildStats *st;
+};
+
+template <class TI, class TO>
+sell_status run_scatter(const ScatterArgs &a, cudaStream_t s) {
+    const TI *vi = static_cast<const TI *>(a.val_in);
+    TO *vo = static_cast<TO *>(a.val);
+    if (a.C % 32 == 0) {
+        const int64_t items = a.Np / 32 + a.nunits * (a.C / 32);
+        k_scatter_tiled<TI, TO><<<(unsigned)((items + kScatterWarps - 1) / kScatterWarps), kScatterWarps * 32, 0, s>>>(
+            a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs, a.lchunk, a.lunit, a.nunits, a.N, a.Np / 32, a.C,
+            a.ncols, vo, a.col, a.st);
+    } else {
+        k_scatter<TI, TO><<<grid_for(a.Np, 256), 256, 0, s>>>(a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs,
+                                                              a.N, a.Np, a.C, a.ncols, vo, a.col, a.st);
     }
     SELL_CUDA_TRY(cudaGetLastError());
     return SELL_OK;
+}
+
+template <class TI>
+sell_status launch_scatter(const ScatterArgs &a, int store, cudaStream_t s) {
+    switch (store) {
+        case SELL_F64: return run_scatter<TI, double>(a, s);
+        case SELL_F32: return run_scatter<TI, float>(a, s);
+        default: return run_scatter<TI, __nv_bfloat16>(a, s);
+    }
 }
 
 int bits_for(unsigned long long v) {  // bits needed to hold 0..v
     int b = 0;
     while (b < 64 && (v >> b) != 0) ++b;
     return b;
+}
+
+// LSD radix sort of the rows by (window, max_rl - rowLen), 8 bits a pass.
+template <class KT>
+sell_status radix_sort(const int32_t *rl, int64_t N, int64_t sigma, int lbits, int bits, int max_rl, int32_t *perm,
+                       const Allocator &al, cudaStream_t s) {
+    const int passes = (bits + 7) / 8;
+    const int64_t ntiles = (N + kRadixTile - 1) / kRadixTile;
+    const uint32_t sg = (uint32_t)std::min<int64_t>(sigma, 0x7FFFFFFF);  // rows are numbered below 2^31
+    DevBuf k0, k1, v1, hist, off;
+    SELL_TRY(k0.alloc(al, N * sizeof(KT), s));
+    SELL_TRY(k1.alloc(al, N * sizeof(KT), s));
+    SELL_TRY(v1.alloc(al, N * sizeof(int32_t), s));
+    SELL_TRY(hist.alloc(al, 256 * ntiles * sizeof(uint32_t), s));
+    SELL_TRY(off.alloc(al, (256 * ntiles + 1) * sizeof(int64_t), s));
+    KT *ka = k0.as<KT>(), *kb = k1.as<KT>();
+    // the values ping-pong between perm and v1 and end in perm
+    int32_t *va = (passes % 2 == 0) ? perm : v1.as<int32_t>();
+    int32_t *vb = (passes % 2 == 0) ? v1.as<int32_t>() : perm;
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+        const unsigned nt = (unsigned)ntiles;
+        uint32_t *hp = hist.as<uint32_t>();
+        if (p == 0) k_radix_hist<KT, true><<<nt, kRadixThreads, 0, s>>>(ka, rl, N, sg, lbits, max_rl, shift, ntiles, hp);
+        else k_radix_hist<KT, false><<<nt, kRadixThreads, 0, s>>>(ka, rl, N, sg, lbits, max_rl, shift, ntiles, hp);
+        SELL_CUDA_TRY(cudaGetLastError());
+        SELL_TRY(scan_exclusive<uint32_t>(hp, 256 * ntiles, off.as<int64_t>(), al, s));
+        const int64_t *op = off.as<int64_t>();
+        if (p == 0)
+            k_radix_scatter<KT, true><<<nt, kRadixThreads, 0, s>>>(ka, va, kb, vb, rl, N, sg, lbits, max_rl, shift,
+                                                                   ntiles, op);
+        else
+            k_radix_scatter<KT, false><<<nt, kRadixThreads, 0, s>>>(ka, va, kb, vb, rl, N, sg, lbits, max_rl, shift,
+                                                                    ntiles, op);
+        SELL_CUDA_TRY(cudaGetLastError());
+        std::swap(ka, kb);
+        std::swap(va, vb);
+    }
+    // after the last swap `va` holds the result and is `perm` by construction
+    return SELL_OK;
 }
 
 sell_status sort_windows(const int32_t *rl, int64_t N, int64_t sigma, int max_rl, int32_t *perm,
@@ -517,35 +855,8 @@ sell_status sort_windows(const int32_t *rl, int64_t N, int64_t sigma, int max_rl
     int wbits = bits_for((unsigned long long)(nwin - 1));
     int total = lbits + wbits;
     if (total > 64) return fail(SELL_EUNSUPPORTED, "sort key wider than 64 bits");
-    int passes = (total + 7) / 8;
-    int64_t ntiles = (N + kRadixTile - 1) / kRadixTile;
-    DevBuf k0, k1, v1, hist, off;
-    SELL_TRY(k0.alloc(al, N * sizeof(unsigned long long), s));
-    SELL_TRY(k1.alloc(al, N * sizeof(unsigned long long), s));
-    SELL_TRY(v1.alloc(al, N * sizeof(int32_t), s));
-    SELL_TRY(hist.alloc(al, 256 * ntiles * sizeof(uint32_t), s));
-    SELL_TRY(off.alloc(al, (256 * ntiles + 1) * sizeof(int64_t), s));
-    unsigned long long *ka = k0.as<unsigned long long>(), *kb = k1.as<unsigned long long>();
-    // the values ping-pong between perm and v1; an odd pass count ends in v1
-    int32_t *va = (passes % 2 == 0) ? perm : v1.as<int32_t>();
-    int32_t *vb = (passes % 2 == 0) ? v1.as<int32_t>() : perm;
-    k_radix_init<<<grid_for(N, 256), 256, 0, s>>>(rl, N, sigma, lbits, max_rl, ka, va);
-    SELL_CUDA_TRY(cudaGetLastError());
-    for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        k_radix_hist<<<(unsigned)ntiles, kRadixThreads, 0, s>>>(ka, N, shift, ntiles,
-                                                               hist.as<uint32_t>());
-        SELL_CUDA_TRY(cudaGetLastError());
-        SELL_TRY(scan_exclusive<uint32_t>(hist.as<uint32_t>(), 1, 256 * ntiles, off.as<int64_t>(),
-                                          al, s));
-        k_radix_scatter<<<(unsigned)ntiles, kRadixThreads, 0, s>>>(ka, va, kb, vb, N, shift, ntiles,
-                                                                   off.as<int64_t>());
-        SELL_CUDA_TRY(cudaGetLastError());
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
-    // after the last swap `va` holds the result and is `perm` by construction
-    return SELL_OK;
+    if (total <= 32) return radix_sort<uint32_t>(rl, N, sigma, lbits, total, max_rl, perm, al, s);
+    return radix_sort<unsigned long long>(rl, N, sigma, lbits, total, max_rl, perm, al, s);
 }
 
 sell_status validate(const sell_csr *A, const sell_opts *o) {
@@ -569,6 +880,16 @@ sell_status validate(const sell_csr *A, const sell_opts *o) {
     int64_t np = (A->nrows + o->C - 1) / o->C * (int64_t)o->C;
     if (np > 0x7FFFFFFFll) return fail(SELL_EINVAL, "sell_build: padded row count exceeds 2^31");
     return SELL_OK;
+}
+
+sell_status malformed(unsigned int err) {
+    std::string m = "sell_build: malformed CRS:";
+    if (err & kErrRpt0) m += " rpt[0] != 0;";
+    if (err & kErrRptOrder) m += " rpt decreasing;";
+    if (err & kErrRptEnd) m += " rpt[nrows] != nnz;";
+    if (err & kErrRowLong) m += " row longer than 2^31-1;";
+    if (err & kErrCol) m += " column index out of range;";
+    return fail(SELL_EINVAL, m);
 }
 
 }  // namespace
@@ -610,28 +931,14 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     SELL_CUDA_TRY(cudaMemsetAsync(stats.p, 0, sizeof(BuildStats), s));
     if (N > 0) {
         SELL_TRY(rl.alloc(al, N * sizeof(int32_t), s));
-        k_rowlen<<<grid_for(N, 256, 152 * 16), 256, 0, s>>>(rpt, N, nnz, rl.as<int32_t>(),
-                                                            stats.as<BuildStats>());
-        SELL_CUDA_TRY(cudaGetLastError());
-    }
-    if (nnz > 0) {
-        k_colcheck<<<grid_for(nnz, 256, 152 * 16), 256, 0, s>>>(col_in, nnz, A->ncols,
-                                                                stats.as<BuildStats>());
+        k_rowlen<<<grid_for(N, 256, 152 * 4), 256, 0, s>>>(rpt, N, nnz, rl.as<int32_t>(), stats.as<BuildStats>());
         SELL_CUDA_TRY(cudaGetLastError());
     }
     BuildStats hs;
     SELL_CUDA_TRY(cudaMemcpyAsync(&hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, s));
     SELL_CUDA_TRY(cudaStreamSynchronize(s));
     if (N == 0 && nnz != 0) hs.err |= kErrRptEnd;
-    if (hs.err) {
-        std::string m = "sell_build: malformed CRS:";
-        if (hs.err & kErrRpt0) m += " rpt[0] != 0;";
-        if (hs.err & kErrRptOrder) m += " rpt decreasing;";
-        if (hs.err & kErrRptEnd) m += " rpt[nrows] != nnz;";
-        if (hs.err & kErrRowLong) m += " row longer than 2^31-1;";
-        if (hs.err & kErrCol) m += " column index out of range;";
-        return fail(SELL_EINVAL, m);
-    }
+    if (hs.err) return malformed(hs.err);
 
     // 3. sorting scope
     DevBuf perm;
@@ -642,64 +949,56 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     }
 
     // 4. chunk lengths (Eq. "max") and sorted row lengths
-    DevBuf srl, cl, cs, inv;
+    DevBuf srl, cl, cs, inv, src;
     if (Np > 0) {
         SELL_TRY(srl.alloc(al, Np * sizeof(int32_t), s));
         SELL_TRY(cl.alloc(al, Nc * sizeof(int32_t), s));
+        SELL_TRY(src.alloc(al, Np * sizeof(int64_t), s));
         SELL_CUDA_TRY(cudaMemsetAsync(cl.p, 0, Nc * sizeof(int32_t), s));
     }
     const bool permute_cols = (o->flags & SELL_BUILD_PERMUTE_COLS) != 0;
     if (permute_cols && N > 0) SELL_TRY(inv.alloc(al, N * sizeof(int32_t), s));
     if (Np > 0) {
         int g = grid_for(Np, 256);
-        k_chunk_len<<<g, 256, 0, s>>>(rl.as<int32_t>(), sorted ? perm.as<int32_t>() : nullptr, N, Np,
-                                      C, srl.as<int32_t>(), cl.as<int32_t>(),
+        k_chunk_len<<<g, 256, 0, s>>>(rl.as<int32_t>(), sorted ? perm.as<int32_t>() : nullptr, rpt, N, Np,
+                                      C, srl.as<int32_t>(), src.as<int64_t>(), cl.as<int32_t>(),
                                       permute_cols ? inv.as<int32_t>() : nullptr);
         SELL_CUDA_TRY(cudaGetLastError());
     }
     // 5. chunk offsets, and the chunks that hold rows longer than kSeg
     SELL_TRY(cs.alloc(al, (Nc + 1) * sizeof(int64_t), s));
-    SELL_TRY(scan_exclusive<int32_t>(cl.as<int32_t>(), C, Nc, cs.as<int64_t>(), al, s));
-    DevBuf lflag, lpos;
+    DevBuf tile, lpos, ubase;
+    ChunkSums total = {0, 0, 0};
     if (Nc > 0) {
-        SELL_TRY(lflag.alloc(al, Nc * sizeof(int32_t), s));
-        SELL_TRY(lpos.alloc(al, (Nc + 1) * sizeof(int64_t), s));
-        k_long_flags<<<grid_for(Nc, 256), 256, 0, s>>>(cl.as<int32_t>(), Nc, lflag.as<int32_t>());
+        // tile sums, then the grand total; the block of tile t adds up the t
+        // tile sums before it (at most 2048)
+        const int64_t per = ((Nc + 2047) / 2048 + kScanThreads - 1) / kScanThreads * kScanThreads;
+        const int64_t nt = (Nc + per - 1) / per;
+        SELL_TRY(tile.alloc(al, (nt + 1) * sizeof(ChunkSums), s));
+        SELL_TRY(lpos.alloc(al, Nc * sizeof(int64_t), s));
+        SELL_TRY(ubase.alloc(al, Nc * sizeof(int64_t), s));
+        ChunkSums *tp = tile.as<ChunkSums>();
+        k_chunk_reduce<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), Nc, per, C, tp);
         SELL_CUDA_TRY(cudaGetLastError());
-        SELL_TRY(scan_exclusive<int32_t>(lflag.as<int32_t>(), 1, Nc, lpos.as<int64_t>(), al, s));
+        k_chunk_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), Nc, per, C, tp, cs.as<int64_t>(),
+                                                            lpos.as<int64_t>(), ubase.as<int64_t>(), tp + nt);
+        SELL_CUDA_TRY(cudaGetLastError());
+        SELL_CUDA_TRY(cudaMemcpyAsync(&total, tp + nt, sizeof(total), cudaMemcpyDeviceToHost, s));
+        SELL_CUDA_TRY(cudaStreamSynchronize(s));
+    } else {
+        SELL_CUDA_TRY(cudaMemsetAsync(cs.p, 0, sizeof(int64_t), s));
     }
-    int64_t stored = 0, nlong = 0;
-    SELL_CUDA_TRY(cudaMemcpyAsync(&stored, cs.as<int64_t>() + Nc, sizeof(int64_t),
-                                  cudaMemcpyDeviceToHost, s));
-    if (Nc > 0)
-        SELL_CUDA_TRY(cudaMemcpyAsync(&nlong, lpos.as<int64_t>() + Nc, sizeof(int64_t),
-                                      cudaMemcpyDeviceToHost, s));
-    SELL_CUDA_TRY(cudaStreamSynchronize(s));
-    DevBuf lchunk, lnseg, lubase, lunit, cnt, cnt2, part, lrow, lmeta;
-    int64_t nunits = 0;
+    const int64_t stored = total.stored, nlong = total.nlong, nunits = total.nunits;
+    DevBuf lchunk, lunit, cnt, cnt2, part, lrow, lmeta;
     if (nlong > 0) {
         SELL_TRY(lchunk.alloc(al, nlong * sizeof(int32_t), s));
-        k_long_compact<<<grid_for(Nc, 256), 256, 0, s>>>(cl.as<int32_t>(), lpos.as<int64_t>(), Nc,
-                                                         lchunk.as<int32_t>());
-        SELL_CUDA_TRY(cudaGetLastError());
-        SELL_TRY(lnseg.alloc(al, nlong * sizeof(int32_t), s));
-        SELL_TRY(lubase.alloc(al, (nlong + 1) * sizeof(int64_t), s));
-        k_long_nseg<<<grid_for(nlong, 256), 256, 0, s>>>(cl.as<int32_t>(), lchunk.as<int32_t>(), nlong,
-                                                         lnseg.as<int32_t>());
-        SELL_CUDA_TRY(cudaGetLastError());
-        SELL_TRY(scan_exclusive<int32_t>(lnseg.as<int32_t>(), 1, nlong, lubase.as<int64_t>(), al, s));
-        SELL_CUDA_TRY(cudaMemcpyAsync(&nunits, lubase.as<int64_t>() + nlong, sizeof(int64_t),
-                                      cudaMemcpyDeviceToHost, s));
-        SELL_CUDA_TRY(cudaStreamSynchronize(s));
         SELL_TRY(lunit.alloc(al, nunits * sizeof(int2), s));
-        k_long_units<<<grid_for(nlong, 256), 256, 0, s>>>(lnseg.as<int32_t>(), lubase.as<int64_t>(), nlong,
-                                                          lunit.as<int2>());
-        SELL_CUDA_TRY(cudaGetLastError());
         SELL_TRY(lrow.alloc(al, (size_t)nlong * C * sizeof(int32_t), s));
         SELL_TRY(lmeta.alloc(al, (size_t)nlong * sizeof(int4), s));
-        k_long_rows<<<grid_for(nlong, 256), 256, 0, s>>>(srl.as<int32_t>(), N, C, lchunk.as<int32_t>(),
-                                                         lnseg.as<int32_t>(), nlong, lrow.as<int32_t>(),
-                                                         lmeta.as<int4>());
+        k_long_lists<<<(unsigned)((Nc + 7) / 8), 256, 0, s>>>(cl.as<int32_t>(), srl.as<int32_t>(),
+                                                                  lpos.as<int64_t>(), ubase.as<int64_t>(), Nc, N, C,
+                                                                  lchunk.as<int32_t>(), lunit.as<int2>(),
+                                                                  lrow.as<int32_t>(), lmeta.as<int4>());
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_TRY(cnt.alloc(al, nlong * C * sizeof(int32_t), s));
         SELL_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, nlong * C * sizeof(int32_t), s));
@@ -708,24 +1007,36 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_TRY(part.alloc(al, (size_t)nunits * C * 8, s));
     }
 
-    // 6. values and columns
+    // 6. values and columns (the column range is checked on the way)
     DevBuf val, col;
     const size_t vs = value_size(o->store_type);
     if (stored > 0) {
         SELL_TRY(val.alloc(al, stored * vs, s));
         SELL_TRY(col.alloc(al, stored * sizeof(int32_t), s));
-        if (A->val_type == SELL_F64)
-            SELL_TRY(launch_scatter<double>(*A, rpt, col_in, val_in, sorted ? perm.as<int32_t>() : nullptr,
-                                            permute_cols ? inv.as<int32_t>() : nullptr,
-                                            srl.as<int32_t>(), cl.as<int32_t>(), cs.as<int64_t>(), Np, C,
-                                            o->store_type, val.p, col.as<int32_t>(), s));
-        else
-            SELL_TRY(launch_scatter<float>(*A, rpt, col_in, val_in, sorted ? perm.as<int32_t>() : nullptr,
-                                           permute_cols ? inv.as<int32_t>() : nullptr,
-                                           srl.as<int32_t>(), cl.as<int32_t>(), cs.as<int64_t>(), Np, C,
-                                           o->store_type, val.p, col.as<int32_t>(), s));
+        ScatterArgs a;
+        a.src = src.as<int64_t>();
+        a.col_in = col_in;
+        a.val_in = val_in;
+        a.inv = permute_cols ? inv.as<int32_t>() : nullptr;
+        a.srl = srl.as<int32_t>();
+        a.cl = cl.as<int32_t>();
+        a.cs = cs.as<int64_t>();
+        a.lchunk = lchunk.as<int32_t>();
+        a.lunit = lunit.as<int2>();
+        a.nunits = nunits;
+        a.N = N;
+        a.Np = Np;
+        a.ncols = A->ncols;
+        a.C = C;
+        a.val = val.p;
+        a.col = col.as<int32_t>();
+        a.st = stats.as<BuildStats>();
+        if (A->val_type == SELL_F64) SELL_TRY(launch_scatter<double>(a, o->store_type, s));
+        else SELL_TRY(launch_scatter<float>(a, o->store_type, s));
+        SELL_CUDA_TRY(cudaMemcpyAsync(&hs.err, &a.st->err, sizeof(hs.err), cudaMemcpyDeviceToHost, s));
     }
     SELL_CUDA_TRY(cudaStreamSynchronize(s));
+    if (hs.err) return malformed(hs.err);
 
     // 7. hand the arrays to the handle
     h->nrows = N;
@@ -803,7 +1114,7 @@ sell_status bulk_plan(sell_matrix *h, int64_t nw, cudaStream_t s) {
         h->wsplit = static_cast<int32_t *>(p);
         SELL_TRY(bss.alloc(al, (Nc + 1) * sizeof(int64_t), s));
         if (Nc > 0) {
-            SELL_TRY(scan_exclusive<int32_t>(bw.as<int32_t>(), 1, Nc, bss.as<int64_t>(), al, s));
+            SELL_TRY(scan_exclusive<int32_t>(bw.as<int32_t>(), Nc, bss.as<int64_t>(), al, s));
         } else {
             SELL_CUDA_TRY(cudaMemsetAsync(bss.p, 0, sizeof(int64_t), s));
         }
