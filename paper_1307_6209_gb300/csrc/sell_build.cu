@@ -41,10 +41,13 @@ constexpr int kRadixThreads = 256;
 constexpr int kRadixRounds = 8;
 constexpr int kRadixTile = kRadixThreads * kRadixRounds;
 
+constexpr int kNopatSlots = 64;  // counters, so that warps rarely meet on one
+
 struct BuildStats {
     unsigned int err;
     int max_rl;
     unsigned long long sumsq;
+    unsigned long long nopat[kNopatSlots];  // stored elements of slices without a column pattern
 };
 enum : unsigned int {
     kErrRpt0 = 1u,
@@ -630,6 +633,13 @@ __global__ void k_scatter(const int64_t *__restrict__ src_of, const int32_t *__r
 // flight: 8 per lane for 8-byte values (235 us; 4: 283 us), 4 for the others
 // (1M banded rows to binary32 80 us; 8: 94 us); a branch around each load
 // instead of a predicate cost up to 60 % more.
+//
+// On the way the warp finds out whether its slice has one column pattern: the
+// entry j of every row lies at (the row's first column) + off[j], with off[j]
+// the same for all rows that have an entry j.  Rows of structured grids away
+// from their boundary and of dense blocks do.  off[j] goes to scol (at
+// offset_start), and sflag[slice] is cleared for slices without a pattern; their
+// stored elements are counted in st->nopat.
 constexpr int kTileCols = 16;
 
 // A read-only load under a predicate, zero otherwise, with no branch around
@@ -660,7 +670,8 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
                 const TI *__restrict__ val_in, const int32_t *__restrict__ inv, const int32_t *__restrict__ srl,
                 const int32_t *__restrict__ cl, const int64_t *__restrict__ cs, const int32_t *__restrict__ lchunk,
                 const int2 *__restrict__ lunit, int64_t nunits, int64_t N, int64_t nslices, int C, int64_t ncols,
-                TO *__restrict__ val, int32_t *__restrict__ col, BuildStats *st) {
+                TO *__restrict__ val, int32_t *__restrict__ col, int32_t *__restrict__ scol,
+                int32_t *__restrict__ sflag, BuildStats *st) {
     // row pitches that keep the column-wise writes of a half-warp off each
     // other's banks
     __shared__ TO tval[kScatterWarps][kTileCols][sizeof(TO) == 8 ? 33 : 34];
@@ -685,7 +696,9 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
     }
     const int64_t slice = c * spc + sl, r = slice * 32 + lane;
     const int64_t cs0 = cs[c];
-    const int j0 = seg * kSeg, j1 = min(cl[c], j0 + kSeg);
+    const int width = cl[c];
+    const int j0 = seg * kSeg, j1 = min(width, j0 + kSeg);
+    const int64_t ostart = offset_start(cs0, width, (int)sl, slice);
     const int len = r < N ? srl[r] : 0;
     const int64_t src = r < N ? src_of[r] : 0;
     const int wmax = __reduce_max_sync(0xffffffffu, len);
@@ -695,6 +708,10 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
         bad |= out;
         return inv && !out ? inv[cidx] : cidx;
     };
+    const int lref = __ffs(__ballot_sync(0xffffffffu, len == wmax)) - 1;
+    int32_t first = seg > 0 && len > 0 ? mapped(col_in[src]) : 0;  // segment 0 has it in its first tile
+    int32_t fref = __shfl_sync(0xffffffffu, first, lref);
+    bool same = true;
     auto load_tile = [&](auto lanes_log2, int jt) {
         constexpr int LG = decltype(lanes_log2)::value;
         constexpr int B = sizeof(TO) == 8 ? 8 : 4;  // loads in flight per lane and array, at most 1 << LG
@@ -730,21 +747,35 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
             else if (rest > 4) load_tile(std::integral_constant<int, 3>(), jt);
             else load_tile(std::integral_constant<int, 2>(), jt);
             __syncwarp();
+            if (jt == 0) {
+                first = tcol[warp][0][lane];
+                fref = __shfl_sync(0xffffffffu, first, lref);
+            }
         }
         const int nj = min(kTileCols, j1 - jt);
+        int32_t myoff = 0;
         int64_t pos = cs0 + (int64_t)jt * C + sl * 32 + lane;
         for (int q = 0; q < nj; ++q, pos += C) {
             if (jt + q < wmax) {
+                const int32_t cc = tcol[warp][q][lane];
                 val[pos] = tval[warp][q][lane];
-                col[pos] = tcol[warp][q][lane];
+                col[pos] = cc;
+                const int32_t off = __shfl_sync(0xffffffffu, cc, lref) - fref;
+                same &= jt + q >= len || cc - first == off;
+                if (lane == q) myoff = off;
             } else {  // columns that only other slices of the chunk reach
                 val[pos] = zero_of<TO>();
                 col[pos] = 0;
             }
         }
+        if (lane < nj) scol[ostart + jt + lane] = myoff;
         __syncwarp();
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&st->err, kErrCol);
+    if (!__all_sync(0xffffffffu, same) && lane == 0) {
+        sflag[slice] = 0;
+        atomicAdd(&st->nopat[w % kNopatSlots], (unsigned long long)(min(wmax, j1) - j0) * 32);
+    }
 }
 
 // Arrays of the format under construction that the scatter reads or writes.
@@ -759,7 +790,7 @@ struct ScatterArgs {
     int64_t nunits, N, Np, ncols;
     int C;
     void *val;
-    int32_t *col;
+    int32_t *col, *scol, *sflag;
     BuildStats *st;
 };
 
@@ -771,7 +802,7 @@ sell_status run_scatter(const ScatterArgs &a, cudaStream_t s) {
         const int64_t items = a.Np / 32 + a.nunits * (a.C / 32);
         k_scatter_tiled<TI, TO><<<(unsigned)((items + kScatterWarps - 1) / kScatterWarps), kScatterWarps * 32, 0, s>>>(
             a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs, a.lchunk, a.lunit, a.nunits, a.N, a.Np / 32, a.C,
-            a.ncols, vo, a.col, a.st);
+            a.ncols, vo, a.col, a.scol, a.sflag, a.st);
     } else {
         k_scatter<TI, TO><<<grid_for(a.Np, 256), 256, 0, s>>>(a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs,
                                                               a.N, a.Np, a.C, a.ncols, vo, a.col, a.st);
@@ -1008,7 +1039,9 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     }
 
     // 6. values and columns (the column range is checked on the way)
-    DevBuf val, col;
+    DevBuf val, col, scol, sflag;
+    bool pattern = false;
+    const bool tiled = C % 32 == 0;
     const size_t vs = value_size(o->store_type);
     if (stored > 0) {
         SELL_TRY(val.alloc(al, stored * vs, s));
@@ -1030,13 +1063,35 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         a.C = C;
         a.val = val.p;
         a.col = col.as<int32_t>();
+        a.scol = a.sflag = nullptr;
+        if (tiled) {
+            SELL_TRY(scol.alloc(al, (stored / 32 + 3 * (Np / 32) + 8) * sizeof(int32_t), s));
+            SELL_TRY(sflag.alloc(al, Np / 32 * sizeof(int32_t), s));
+            SELL_CUDA_TRY(cudaMemsetAsync(sflag.p, 1, Np / 32 * sizeof(int32_t), s));  // any non-zero word: a pattern
+            a.scol = scol.as<int32_t>();
+            a.sflag = sflag.as<int32_t>();
+        }
         a.st = stats.as<BuildStats>();
         if (A->val_type == SELL_F64) SELL_TRY(launch_scatter<double>(a, o->store_type, s));
         else SELL_TRY(launch_scatter<float>(a, o->store_type, s));
-        SELL_CUDA_TRY(cudaMemcpyAsync(&hs.err, &a.st->err, sizeof(hs.err), cudaMemcpyDeviceToHost, s));
+        BuildStats end;
+        SELL_CUDA_TRY(cudaMemcpyAsync(&end, a.st, sizeof(end), cudaMemcpyDeviceToHost, s));
+        SELL_CUDA_TRY(cudaStreamSynchronize(s));
+        if (end.err) return malformed(end.err);
+        // The products take the offsets where they save column bytes: at least
+        // half of the stored elements in slices with a pattern.  (Rows of one
+        // entry have a trivial one; a slice without one reads its columns.)
+        unsigned long long nopat = 0;
+        for (unsigned long long n : end.nopat) nopat += n;
+        // The kernel loads offsets and prefetches values in 16-byte units.
+        pattern = tiled && 2 * nopat <= (unsigned long long)stored &&
+                  ((uintptr_t)val.p | (uintptr_t)scol.p) % 16 == 0;
+    }
+    if (!pattern) {
+        scol.reset();
+        sflag.reset();
     }
     SELL_CUDA_TRY(cudaStreamSynchronize(s));
-    if (hs.err) return malformed(hs.err);
 
     // 7. hand the arrays to the handle
     h->nrows = N;
@@ -1062,7 +1117,10 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     h->nunits = nunits;
     h->part_k = nunits > 0 ? 1 : 0;
     h->device_bytes = val.bytes + col.bytes + cs.bytes + cl.bytes + srl.bytes + perm.bytes + lchunk.bytes +
-                      lunit.bytes + cnt.bytes + cnt2.bytes + part.bytes + lrow.bytes + lmeta.bytes;
+                      lunit.bytes + cnt.bytes + cnt2.bytes + part.bytes + lrow.bytes + lmeta.bytes +
+                      scol.bytes + sflag.bytes;
+    h->scol = (int32_t *)scol.release_ownership();
+    h->sflag = (int32_t *)sflag.release_ownership();
     h->lchunk = (int32_t *)lchunk.release_ownership();
     h->lunit = (int2 *)lunit.release_ownership();
     h->lrow = (int32_t *)lrow.release_ownership();

@@ -8,7 +8,6 @@
 #include <stdint.h>
 
 namespace sell {
-
 // Entries per segment of a long row.  Part of the numerics: a row longer than
 // kSeg is summed segment by segment (sell_rowdot.cuh), so changing it changes
 // the rounding of long rows.
@@ -16,6 +15,15 @@ constexpr int kSeg = 64;
 // Segments per group of the two-level fold of very long rows (more than
 // kSeg * kSuper = 16384 entries); also part of the numerics.
 constexpr int kSuper = 256;
+
+// Where the column offsets of a slice (32 rows) begin in scol: every slice
+// takes its chunk's width, and starts at a multiple of four values so that
+// four offsets are one 16-byte load.  The three values of slack per slice
+// make room for the rounding: (a + 3g + 3) & ~3 grows by at least the width
+// from one slice to the next.
+__host__ __device__ __forceinline__ int64_t offset_start(int64_t cs0, int32_t width, int s, int64_t slice) {
+    return ((cs0 >> 5) + (int64_t)s * width + 3 * slice + 3) & ~(int64_t)3;
+}
 
 // --------------------------------------------------------- device helpers
 // Streaming loads for data touched once per product (val/col): do not allocate
@@ -25,6 +33,11 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
     uint64_t p;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
+}
+
+// Ask L2 for `bytes` (a multiple of 16) at p (16-byte aligned), one request.
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes, uint64_t pol) {
+    asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p), "r"(bytes), "l"(pol));
 }
 
 __device__ __forceinline__ double ld_stream(const double *ptr, uint64_t pol) {

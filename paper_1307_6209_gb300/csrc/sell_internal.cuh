@@ -111,6 +111,10 @@ struct sell_matrix {
     int32_t *srl = nullptr;    // nchunks * C, length of each sorted row
     int32_t *perm = nullptr;   // nrows, sorted -> original (null: identity)
     int32_t *lchunk = nullptr; // nlong chunks holding rows longer than kSeg
+    // column offsets of slices with one column pattern (sell_build.cu
+    // k_scatter_tiled): about stored / 32 offsets and one flag per 32 rows; null
+    // unless most of the matrix lies in such slices
+    int32_t *scol = nullptr, *sflag = nullptr;
     int64_t nlong = 0;
     int2 *lunit = nullptr;     // nunits long-row work units {long chunk, segment}
     int32_t *lrow = nullptr;   // nlong * C lanes of each long chunk's long rows

@@ -29,6 +29,12 @@
 
 namespace sell {
 
+// The column offsets of slices with one column pattern, their flags, and the
+// chunk widths that place them (offset_start).
+struct Pattern {
+    const int32_t *off, *flag, *cl;
+};
+
 template <class VT> struct XType;
 template <> struct XType<double> { using T = double; };
 template <> struct XType<float> { using T = float; };
@@ -124,9 +130,7 @@ __device__ __forceinline__ void ld_x32(const double *p, double *v) {
 // (16-byte vector loads), 0 otherwise (one load per value); bits 2-3 hold the
 // same for Y (store_y).  The values loaded are the same in every case.
 template <int K, class XT>
-__device__ __forceinline__ void load_x(const XT *__restrict__ X, int64_t ldx, int32_t ci, int vec,
-                                       XT (&xv)[K]) {
-    const XT *p = X + (int64_t)ci * ldx;
+__device__ __forceinline__ void load_x_at(const XT *__restrict__ p, int vec, XT (&xv)[K]) {
     vec &= 3;
     if constexpr (K == 1) {
         xv[0] = __ldg(p);
@@ -159,6 +163,11 @@ __device__ __forceinline__ void load_x(const XT *__restrict__ X, int64_t ldx, in
             for (int q = 0; q < K; ++q) xv[q] = __ldg(p + q);
         }
     }
+}
+
+template <int K, class XT>
+__device__ __forceinline__ void load_x(const XT *__restrict__ X, int64_t ldx, int32_t ci, int vec, XT (&xv)[K]) {
+    load_x_at<K>(X + (int64_t)ci * ldx, vec, xv);
 }
 
 // 32 bytes of Y at p (32-byte aligned) in one 256-bit store or load.
@@ -356,6 +365,136 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
     }
 }
 
+// The same chain for a row of a slice with one column pattern: entry j lies
+// in column first + op[j], op the same for the whole warp (16-byte loads that
+// all lanes share).  U is 2 or a multiple of 4, j0 a multiple of U; CT is the chunk height
+// where it is known at compile time (the strides become constants of the
+// load instructions), else 0.
+template <class VT, class XT, int K, int U, bool PIPE, int CT, class Acc>
+__device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restrict__ vp,
+                                              const int32_t *__restrict__ op, int32_t first, int C, int j0, int j1,
+                                              const XT *__restrict__ X, int64_t ldx, int vec, uint64_t pol) {
+    const int64_t stride = CT ? CT : C;
+    // the row pitch of X in bytes fits 31 bits (run_pattern), so that a row's
+    // address is one multiply-add
+    const char *xp = reinterpret_cast<const char *>(X + (int64_t)first * ldx);
+    const int32_t pitch = (int32_t)(ldx * (int64_t)sizeof(XT));
+    op += j0;
+    vp += (int64_t)j0 * stride;
+    constexpr int XB = K >= 8 && U > 2 ? 2 : U;  // rows of X in flight
+    int j = j0;
+    auto group = [&](const VT (&v)[U], const int32_t (&o)[U], int n) {
+#pragma unroll
+        for (int b = 0; b < U; b += XB) {
+            XT xv[XB][K];
+#pragma unroll
+            for (int u = 0; u < XB; ++u)
+                if (b + u < n)
+                    load_x_at<K>(reinterpret_cast<const XT *>(xp + (int64_t)o[b + u] * pitch), vec, xv[u]);
+#pragma unroll
+            for (int u = 0; u < XB; ++u) {
+                if (b + u < n) {
+                    const XT a = widen(v[b + u]);
+#pragma unroll
+                    for (int q = 0; q < K; ++q) acc[q].add(a, xv[u][q]);
+                }
+            }
+        }
+    };
+    auto offsets = [&](int32_t (&o)[U], int at) {
+        if constexpr (U % 4 == 0) {
+#pragma unroll
+            for (int u = 0; u < U; u += 4) {
+                const int4 t = __ldg(reinterpret_cast<const int4 *>(op + at + u));
+                o[u] = t.x;
+                o[u + 1] = t.y;
+                o[u + 2] = t.z;
+                o[u + 3] = t.w;
+            }
+        } else {
+            const int2 t = __ldg(reinterpret_cast<const int2 *>(op + at));
+            o[0] = t.x;
+            o[1] = t.y;
+        }
+    };
+    if constexpr (PIPE) {
+        VT v[U], vn[U];
+        int32_t o[U], on[U];
+        if (j < j1) {
+            offsets(o, 0);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + u < j1) v[u] = ld_stream(vp + u * stride, pol);
+        }
+        for (; j + U < j1; j += U) {
+            offsets(on, U);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + U + u < j1) vn[u] = ld_stream(vp + (U + u) * stride, pol);
+            group(v, o, U);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                v[u] = vn[u];
+                o[u] = on[u];
+            }
+            vp += U * stride;
+            op += U;
+        }
+        if (j < j1) group(v, o, j1 - j);
+    } else {
+        for (; j + U <= j1; j += U) {
+            VT v[U];
+            int32_t o[U];
+            offsets(o, 0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = ld_stream(vp + u * stride, pol);
+            group(v, o, U);
+            vp += U * stride;
+            op += U;
+        }
+        if (j < j1) {
+            VT v[U];
+            int32_t o[U];
+            offsets(o, 0);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + u < j1) v[u] = ld_stream(vp + u * stride, pol);
+            group(v, o, j1 - j);
+        }
+    }
+}
+
+// The chain over entries j0..j1-1 of sorted row r = lane l of chunk c.
+// PAT: the matrix has slices with one column pattern.
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT>
+__device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ val, const int32_t *__restrict__ col,
+                                          const int64_t *__restrict__ cs, const Pattern &pt, int C, int64_t r,
+                                          int64_t c, int l, int j0, int j1, const XT *__restrict__ X, int64_t ldx,
+                                          int vec, uint64_t pol) {
+    const int64_t cs0 = cs[c];
+    const int64_t base = cs0 + l;
+    if constexpr (PAT) {
+        // one request brings the warp's values to L2 (the first lane's row
+        // stands for all), so that the loads below wait for L2 and not for HBM
+        constexpr bool PREFETCH = sizeof(XT) == 4 || K < 4;  // wider binary64 products are bound by the FP64 pipe
+        const int32_t width = pt.cl[c];
+        const int n = j1 - j0;
+        const int64_t at = cs0 + (int64_t)j0 * C + (int64_t)(l & ~31) * n;
+        const bool ask = PREFETCH && (l & 31) == 0 && n > 0;
+        if (ask) prefetch_l2(val + at, (uint32_t)(n * 32 * sizeof(VT)), pol);
+        if (pt.flag[r >> 5]) {
+            if (n <= 0) return;
+            const int32_t first = __ldg(col + base);
+            const int32_t *op = pt.off + offset_start(cs0, width, l >> 5, r >> 5);
+            if (C == 32) chain_pattern<VT, XT, K, U, PIPE, 32, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+            else chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+            return;
+        }
+        if (ask) prefetch_l2(col + at, (uint32_t)(n * 128), pol);
+    }
+    chain<VT, XT, K, U, PIPE, Acc>(acc, val + base, col + base, C, j0, j1, X, ldx, vec, pol);
+}
+
 // Fold `count` partials of lane l, found at units base, base + stride, ...,
 // in that order (loads issued FB at a time, folds strictly in order).
 template <int K, class Acc>
@@ -394,10 +533,13 @@ __device__ __forceinline__ void fold_partials(const Acc *part, int64_t base, int
 // that completes the group (its result replaces the group's first partial),
 // then the thread that completes the last group folds the group results in
 // order.  Either way the result depends only on the row's entries.
-template <class VT, class XT, int K, int U, bool PIPE, class Acc>
+//
+// PAT: the matrix has slices with one column pattern (pt; C is a multiple of
+// 32).
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT = false>
 __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const int32_t *__restrict__ srl,
-                                          const int32_t *__restrict__ perm, const int32_t *__restrict__ lchunk,
+                                          const int32_t *__restrict__ perm, const Pattern &pt, const int32_t *__restrict__ lchunk,
                                           const int2 *__restrict__ lunit, const int4 *__restrict__ lmeta,
                                           const int32_t *__restrict__ lrow, Acc *part, int32_t *cnt,
                                           int32_t *cnt2, const XT *__restrict__ X, int64_t ldx, XT *Y,
@@ -430,9 +572,8 @@ __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int3
     Acc acc[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) acc[q].init((s == 0 && accumulate) ? Y[out * ldy + q] : XT(0));
-    const int64_t base = cs[c] + l;
-    chain<VT, XT, K, U, PIPE, Acc>(acc, val + base, col + base, C, s * kSeg, min(L, (s + 1) * kSeg), X, ldx,
-                                   vec & 3, pol);
+    row_chain<VT, XT, K, U, PIPE, Acc, PAT>(acc, val, col, cs, pt, C, r, c, l, s * kSeg, min(L, (s + 1) * kSeg), X,
+                                            ldx, vec & 3, pol);
     using PT = typename PartOf<Acc>::T;
     PT *pp = reinterpret_cast<PT *>(part);
 #pragma unroll
@@ -467,18 +608,17 @@ __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int3
 }
 
 // The thread's own row when it is short (L <= kSeg); long rows return.
-template <class VT, class XT, int K, int U, bool PIPE, class Acc>
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT = false>
 __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const int32_t *__restrict__ srl,
-                                          const int32_t *__restrict__ perm, const XT *__restrict__ X,
+                                          const int32_t *__restrict__ perm, const Pattern &pt, const XT *__restrict__ X,
                                           int64_t ldx, XT *Y, int64_t ldy, int C, int64_t r, int accumulate,
                                           int vec, uint64_t pol) {
     const int L = srl[r];
     if (L > kSeg) return;
-    const int64_t c = r / C;
-    const int l = (int)(r - c * C);
+    const uint32_t c = (uint32_t)r / (uint32_t)C;  // padded row numbers stay below 2^31
+    const int l = (int)((uint32_t)r - c * (uint32_t)C);
     const int64_t out = perm ? (int64_t)perm[r] : r;
-    const int64_t base = cs[c] + l;
     Acc acc[K];
     if (accumulate) {
         XT y0[K];
@@ -489,7 +629,7 @@ __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int3
 #pragma unroll
         for (int q = 0; q < K; ++q) acc[q].init(XT(0));
     }
-    chain<VT, XT, K, U, PIPE, Acc>(acc, val + base, col + base, C, 0, L, X, ldx, vec & 3, pol);
+    row_chain<VT, XT, K, U, PIPE, Acc, PAT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec & 3, pol);
     XT yo[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) yo[q] = acc[q].result();
