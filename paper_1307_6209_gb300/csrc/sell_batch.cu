@@ -97,7 +97,7 @@ __device__ __forceinline__ void batch_unit(const LaunchParams &lp) {
         const int64_t v = first + threadIdx.x;
         if (v < P.long_threads)
             long_unit<VT, XT, K, U, PIPE, AccL>(static_cast<const VT *>(P.val), P.col, P.cs, P.srl, P.perm,
-                                         Pattern{}, P.lchunk, P.lunit, P.lmeta, P.lrow, static_cast<AccL *>(P.part), P.cnt, P.cnt2,
+                                         P.lchunk, P.lunit, P.lmeta, P.lrow, static_cast<AccL *>(P.part), P.cnt, P.cnt2,
                                          static_cast<const XT *>(P.X),
                                          P.ldx, static_cast<XT *>(P.Y), P.ldy, P.N, P.C, v, P.acc, P.vec, pol);
         return;

@@ -47,7 +47,7 @@ struct BuildStats {
     unsigned int err;
     int max_rl;
     unsigned long long sumsq;
-    unsigned long long nopat[kNopatSlots];  // stored elements of slices without a column pattern
+    unsigned long long nopat[kNopatSlots];  // entries in slices without a column pattern
 };
 enum : unsigned int {
     kErrRpt0 = 1u,
@@ -361,24 +361,39 @@ sell_status scan_exclusive(const T *in, int64_t n, int64_t *out, const Allocator
     return SELL_OK;
 }
 
-// The three sums over the chunks in one scan: chunk offsets (C * cl), long
-// chunks (cl > kSeg) and their segments (ceil(cl / kSeg) each).
+// The sums over the chunks in one scan: chunk offsets (C * cl), long chunks
+// (cl > kSeg), their segments (ceil(cl / kSeg) each), the virtual warps of
+// sell_long.cuh and those of them with packed entries.  nlr[c] = rows of chunk c longer than kSeg.
 struct ChunkSums {
-    int64_t stored, nlong, nunits;
+    int64_t stored, nlong, nunits, nwork, npack;
     __device__ __forceinline__ ChunkSums &operator+=(const ChunkSums &o) {
         stored += o.stored;
         nlong += o.nlong;
         nunits += o.nunits;
+        nwork += o.nwork;
+        npack += o.npack;
         return *this;
     }
 };
-__device__ __forceinline__ ChunkSums sums_of(int32_t cl, int C) {
-    const bool lg = cl > kSeg;
-    return {(int64_t)C * cl, lg ? 1 : 0, lg ? (cl - 1) / kSeg + 1 : 0};  // no overflow near 2^31
+// Whether a chunk with m long rows deals their segments out one row after
+// another (mode 1 of k_long_lists).
+__device__ __forceinline__ bool few_long(int m, int C) { return 8 * (int64_t)m <= C; }
+
+__device__ __forceinline__ ChunkSums sums_of(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr,
+                                             int64_t c, int C) {
+    const int32_t w = cl[c];
+    if (w <= kSeg) return {(int64_t)C * w, 0, 0, 0, 0};
+    const int64_t nseg = (w - 1) / kSeg + 1;  // no overflow near 2^31
+    const int m = nlr[c];
+    if (C % 32) return {(int64_t)C * w, 1, nseg, 0, 0};
+    if (!few_long(m, C)) return {(int64_t)C * w, 1, nseg, nseg * (C / 32), 0};
+    const int64_t work = (m * nseg + 31) / 32;
+    return {(int64_t)C * w, 1, nseg, work, work};
 }
 __device__ __forceinline__ ChunkSums shfl_up(const ChunkSums &v, int o) {
     return {__shfl_up_sync(0xffffffffu, v.stored, o), __shfl_up_sync(0xffffffffu, v.nlong, o),
-            __shfl_up_sync(0xffffffffu, v.nunits, o)};
+            __shfl_up_sync(0xffffffffu, v.nunits, o), __shfl_up_sync(0xffffffffu, v.nwork, o),
+            __shfl_up_sync(0xffffffffu, v.npack, o)};
 }
 // Inclusive scan over the block (1024 threads); *tot = the block's total.
 __device__ __forceinline__ ChunkSums block_inclusive(ChunkSums v, ChunkSums *wt) {
@@ -405,24 +420,26 @@ __device__ __forceinline__ ChunkSums block_inclusive(ChunkSums v, ChunkSums *wt)
 
 // Sums of tiles of `per` chunks (a multiple of 1024), one tile per block.
 __global__ void __launch_bounds__(kScanThreads)
-k_chunk_reduce(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, ChunkSums *__restrict__ tile) {
+k_chunk_reduce(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, int64_t Nc, int64_t per, int C,
+               ChunkSums *__restrict__ tile) {
     __shared__ ChunkSums wt[32];
     const int64_t c0 = blockIdx.x * per, c1 = min(Nc, c0 + per);
-    ChunkSums v = {0, 0, 0};
-    for (int64_t c = c0 + threadIdx.x; c < c1; c += kScanThreads) v += sums_of(cl[c], C);
+    ChunkSums v = {0, 0, 0, 0, 0};
+    for (int64_t c = c0 + threadIdx.x; c < c1; c += kScanThreads) v += sums_of(cl, nlr, c, C);
     v = block_inclusive(v, wt);
     if (threadIdx.x == kScanThreads - 1) tile[blockIdx.x] = v;
 }
 
-// cs, and for the long chunks their index and first unit in lpos/ubase; the
-// totals go to cs[Nc] and *total.  tile: the tile sums.
+// cs, and for the long chunks their index, first unit and first virtual warp
+// (and first packed one) in lpos/ubase/wbase; the totals go to cs[Nc] and *total.  tile: the tile sums.
 __global__ void __launch_bounds__(kScanThreads)
-k_chunk_apply(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, const ChunkSums *__restrict__ tile,
+k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, int64_t Nc, int64_t per, int C,
+              const ChunkSums *__restrict__ tile,
               int64_t *__restrict__ cs, int64_t *__restrict__ lpos, int64_t *__restrict__ ubase,
-              ChunkSums *__restrict__ total) {
+              longlong2 *__restrict__ wbase, ChunkSums *__restrict__ total) {
     __shared__ ChunkSums wt[32];
     __shared__ ChunkSums before;
-    ChunkSums s = {0, 0, 0};
+    ChunkSums s = {0, 0, 0, 0, 0};
     for (int64_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) s += tile[i];
     s = block_inclusive(s, wt);
     if (threadIdx.x == kScanThreads - 1) before = s;
@@ -430,13 +447,14 @@ k_chunk_apply(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, co
     const int64_t c1 = min(Nc, (blockIdx.x + 1) * per);
     for (int64_t c0 = blockIdx.x * per; c0 < c1; c0 += kScanThreads) {
         const int64_t c = c0 + threadIdx.x;
-        const ChunkSums own = sums_of(c < c1 ? cl[c] : 0, C);
+        const ChunkSums own = c < c1 ? sums_of(cl, nlr, c, C) : ChunkSums{0, 0, 0, 0, 0};
         ChunkSums v = block_inclusive(own, wt);
         v += before;
         if (c < c1) {
             cs[c] = v.stored - own.stored;
             lpos[c] = v.nlong - own.nlong;
             ubase[c] = v.nunits - own.nunits;
+            wbase[c] = make_longlong2(v.nwork - own.nwork, v.npack - own.npack);
             if (c == Nc - 1) {
                 cs[Nc] = v.stored;
                 *total = v;
@@ -454,7 +472,8 @@ k_chunk_apply(const int32_t *__restrict__ cl, int64_t Nc, int64_t per, int C, co
 // perm, rpt) before a row's entries.
 __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__restrict__ perm,
                             const int64_t *__restrict__ rpt, int64_t N, int64_t Np, int C, int32_t *__restrict__ srl,
-                            int64_t *__restrict__ src, int32_t *__restrict__ cl, int32_t *__restrict__ inv) {
+                            int64_t *__restrict__ src, int32_t *__restrict__ cl, int32_t *__restrict__ nlr,
+                            int32_t *__restrict__ inv) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool warp_chunks = (C % 32) == 0;
     // the loop trip count is uniform across a warp because Np is a multiple of
@@ -475,9 +494,14 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
         if (warp_chunks) {
             int32_t m = len;
             for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (live && (threadIdx.x & 31) == 0 && m > 0) atomicMax(&cl[r / C], m);
+            const int nl = __popc(__ballot_sync(0xffffffffu, len > kSeg));
+            if (live && (threadIdx.x & 31) == 0 && m > 0) {
+                atomicMax(&cl[r / C], m);
+                if (nl) atomicAdd(&nlr[r / C], nl);
+            }
         } else if (live && len > 0) {
             atomicMax(&cl[r / C], len);
+            if (len > kSeg) atomicAdd(&nlr[r / C], 1);
         }
     }
 }
@@ -495,8 +519,9 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
 // lane of the row), so the results do not depend on the mode.
 __global__ void __launch_bounds__(256)
 k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, const int64_t *__restrict__ lpos,
-             const int64_t *__restrict__ ubase, int64_t Nc, int64_t N, int C, int32_t *__restrict__ lchunk,
-             int2 *__restrict__ lunit, int32_t *__restrict__ lrow, int4 *__restrict__ lmeta) {
+             const int64_t *__restrict__ ubase, const longlong2 *__restrict__ wbase, const int64_t *__restrict__ cs, int64_t Nc, int64_t N, int C,
+             int32_t *__restrict__ lchunk, int2 *__restrict__ lunit, int32_t *__restrict__ lrow,
+             int4 *__restrict__ lmeta, LongWork *__restrict__ lwork) {
     const int lane = threadIdx.x & 31;
     const int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int32_t width = c < Nc ? cl[c] : 0;
@@ -512,9 +537,26 @@ k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, co
         if (lg) lrow[i * C + m + __popc(hit & ((1u << lane) - 1u))] = l0 + lane;
         m += __popc(hit);
     }
+    const bool few = few_long(m, C);
+    if (lwork) {
+        const int64_t n = few ? ((int64_t)m * nseg + 31) / 32 : (int64_t)nseg * (C / 32);
+        const longlong2 wb = wbase[c];
+        for (int64_t k = lane; k < n; k += 32) {
+            LongWork wk;
+            wk.lc = (int32_t)i;
+            wk.c = (int32_t)c;
+            wk.nseg = nseg;
+            wk.m = few ? m : -1;
+            const int sl = (int)(k % (C / 32)), sg = (int)(k / (C / 32));
+            wk.base = few ? (wb.y + k) * (kSeg * 32) : cs[c] + (int64_t)sg * kSeg * C + sl * 32;
+            wk.i = (int32_t)k;
+            wk.u0 = (int32_t)u;
+            lwork[wb.x + k] = wk;
+        }
+    }
     if (lane == 0) {
         lchunk[i] = (int32_t)c;
-        lmeta[i] = make_int4(m, 8 * m <= C ? 1 : 0, nseg, 0);
+        lmeta[i] = make_int4(m, few ? 1 : 0, nseg, 0);
     }
 }
 
@@ -617,7 +659,8 @@ __global__ void k_scatter(const int64_t *__restrict__ src_of, const int32_t *__r
 }
 
 // Chunk heights of a multiple of 32: one warp per slice (32 consecutive sorted
-// rows) and kSeg stored columns, kTileCols of them at a time.  The warp reads
+// rows) and kSeg stored columns, kTileCols of them at a time (and one per
+// virtual warp with packed entries, sell_long.cuh).  The warp reads
 // the entries row by row -- 16 consecutive entries of two rows per load (4 or
 // 8 of more rows where the rows are short), so a row's bytes are read once and
 // in whole sectors -- into a shared tile, and writes the tile column by column
@@ -639,7 +682,7 @@ __global__ void k_scatter(const int64_t *__restrict__ src_of, const int32_t *__r
 // the same for all rows that have an entry j.  Rows of structured grids away
 // from their boundary and of dense blocks do.  off[j] goes to scol (at
 // offset_start), and sflag[slice] is cleared for slices without a pattern; their
-// stored elements are counted in st->nopat.
+// entries are counted in st->nopat.
 constexpr int kTileCols = 16;
 
 // A read-only load under a predicate, zero otherwise, with no branch around
@@ -669,9 +712,10 @@ __global__ void __launch_bounds__(kScatterWarps * 32)
 k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ col_in,
                 const TI *__restrict__ val_in, const int32_t *__restrict__ inv, const int32_t *__restrict__ srl,
                 const int32_t *__restrict__ cl, const int64_t *__restrict__ cs, const int32_t *__restrict__ lchunk,
-                const int2 *__restrict__ lunit, int64_t nunits, int64_t N, int64_t nslices, int C, int64_t ncols,
-                TO *__restrict__ val, int32_t *__restrict__ col, int32_t *__restrict__ scol,
-                int32_t *__restrict__ sflag, BuildStats *st) {
+                const int2 *__restrict__ lunit, const int32_t *__restrict__ lrow, const LongWork *__restrict__ lwork,
+                int64_t nunits, int64_t nlwork, int64_t N, int64_t nslices, int C, int64_t ncols,
+                TO *__restrict__ val, int32_t *__restrict__ col, TO *__restrict__ lval, int32_t *__restrict__ lcol,
+                int32_t *__restrict__ scol, int32_t *__restrict__ sflag, BuildStats *st) {
     // row pitches that keep the column-wise writes of a half-warp off each
     // other's banks
     __shared__ TO tval[kScatterWarps][kTileCols][sizeof(TO) == 8 ? 33 : 34];
@@ -679,28 +723,50 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t w = blockIdx.x * (int64_t)kScatterWarps + warp;
     const uint32_t spc = (uint32_t)C / 32;  // slices per chunk
-    int64_t c;
-    uint32_t sl;
-    int seg = 0;
-    if (w < nslices) {
-        c = (uint32_t)w / spc;
-        sl = (uint32_t)w % spc;
-    } else {
-        const int64_t i = w - nslices;
-        if (i >= nunits * spc) return;
-        const int2 us = lunit[i / spc];
-        seg = us.y;
-        if (seg == 0) return;  // the slice's own warp has the first segment
-        sl = (uint32_t)(i % spc);
-        c = lchunk[us.x];
+    const int64_t npieces = nslices + nunits * spc;
+    int64_t slice = 0, src = 0, at, ostart = 0;  // at: where column j0 of the piece begins
+    int seg = 0, len, j0 = 0, j1 = kSeg, stride = 32;
+    const bool pack = w >= npieces;
+    if (!pack) {
+        int64_t c;
+        uint32_t sl;
+        if (w < nslices) {
+            c = (uint32_t)w / spc;
+            sl = (uint32_t)w % spc;
+        } else {
+            const int64_t i = w - nslices;
+            const int2 us = lunit[i / spc];
+            seg = us.y;
+            if (seg == 0) return;  // the slice's own warp has the first segment
+            sl = (uint32_t)(i % spc);
+            c = lchunk[us.x];
+        }
+        slice = c * spc + sl;
+        const int64_t r = slice * 32 + lane, cs0 = cs[c];
+        const int width = cl[c];
+        len = r < N ? srl[r] : 0;
+        src = r < N ? src_of[r] : 0;
+        j0 = seg * kSeg;
+        j1 = min(width, j0 + kSeg);
+        stride = C;
+        at = cs0 + (int64_t)j0 * C + sl * 32;
+        ostart = offset_start(cs0, width, (int)sl, slice);
+    } else {  // a virtual warp of a chunk with few long rows: lane t's segment as a row of its own
+        if (w - npieces >= nlwork) return;
+        const LongWork wk = lwork[w - npieces];
+        if (wk.m < 0) return;
+        const int64_t i = (int64_t)wk.i * 32 + lane, k = i / wk.nseg;
+        len = 0;
+        if (k < wk.m) {
+            const int64_t r = (int64_t)wk.c * C + lrow[(int64_t)wk.lc * C + k];
+            const int s0 = (int)(i - k * wk.nseg) * kSeg;
+            len = max(0, min(srl[r] - s0, kSeg));
+            src = src_of[r] + s0;
+        }
+        at = wk.base;
+        val = lval;
+        col = lcol;
     }
-    const int64_t slice = c * spc + sl, r = slice * 32 + lane;
-    const int64_t cs0 = cs[c];
-    const int width = cl[c];
-    const int j0 = seg * kSeg, j1 = min(width, j0 + kSeg);
-    const int64_t ostart = offset_start(cs0, width, (int)sl, slice);
-    const int len = r < N ? srl[r] : 0;
-    const int64_t src = r < N ? src_of[r] : 0;
     const int wmax = __reduce_max_sync(0xffffffffu, len);
     bool bad = false;
     auto mapped = [&](int32_t cidx) {
@@ -754,8 +820,8 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
         }
         const int nj = min(kTileCols, j1 - jt);
         int32_t myoff = 0;
-        int64_t pos = cs0 + (int64_t)jt * C + sl * 32 + lane;
-        for (int q = 0; q < nj; ++q, pos += C) {
+        int64_t pos = at + (int64_t)(jt - j0) * stride + lane;
+        for (int q = 0; q < nj; ++q, pos += stride) {
             if (jt + q < wmax) {
                 const int32_t cc = tcol[warp][q][lane];
                 val[pos] = tval[warp][q][lane];
@@ -768,13 +834,16 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
                 col[pos] = 0;
             }
         }
-        if (lane < nj) scol[ostart + jt + lane] = myoff;
+        if (lane < nj && !pack) scol[ostart + jt + lane] = myoff;
         __syncwarp();
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&st->err, kErrCol);
-    if (!__all_sync(0xffffffffu, same) && lane == 0) {
-        sflag[slice] = 0;
-        atomicAdd(&st->nopat[w % kNopatSlots], (unsigned long long)(min(wmax, j1) - j0) * 32);
+    if (!pack && !__all_sync(0xffffffffu, same)) {
+        const unsigned n = __reduce_add_sync(0xffffffffu, (unsigned)max(0, min(len, j1) - j0));
+        if (lane == 0) {
+            sflag[slice] = 0;
+            atomicAdd(&st->nopat[w % kNopatSlots], (unsigned long long)n);
+        }
     }
 }
 
@@ -787,9 +856,12 @@ struct ScatterArgs {
     const int64_t *cs;
     const int32_t *lchunk;
     const int2 *lunit;
-    int64_t nunits, N, Np, ncols;
+    const int32_t *lrow;
+    const LongWork *lwork;
+    int64_t nunits, nlwork, N, Np, ncols;
     int C;
-    void *val;
+    void *val, *lval;
+    int32_t *lcol;
     int32_t *col, *scol, *sflag;
     BuildStats *st;
 };
@@ -799,10 +871,11 @@ sell_status run_scatter(const ScatterArgs &a, cudaStream_t s) {
     const TI *vi = static_cast<const TI *>(a.val_in);
     TO *vo = static_cast<TO *>(a.val);
     if (a.C % 32 == 0) {
-        const int64_t items = a.Np / 32 + a.nunits * (a.C / 32);
+        const int64_t items = a.Np / 32 + a.nunits * (a.C / 32) + (a.lval ? a.nlwork : 0);
         k_scatter_tiled<TI, TO><<<(unsigned)((items + kScatterWarps - 1) / kScatterWarps), kScatterWarps * 32, 0, s>>>(
-            a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs, a.lchunk, a.lunit, a.nunits, a.N, a.Np / 32, a.C,
-            a.ncols, vo, a.col, a.scol, a.sflag, a.st);
+            a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs, a.lchunk, a.lunit, a.lrow, a.lwork,
+            a.nunits, a.nlwork, a.N, a.Np / 32, a.C, a.ncols, vo, a.col, static_cast<TO *>(a.lval), a.lcol, a.scol,
+            a.sflag, a.st);
     } else {
         k_scatter<TI, TO><<<grid_for(a.Np, 256), 256, 0, s>>>(a.src, a.col_in, vi, a.inv, a.srl, a.cl, a.cs,
                                                               a.N, a.Np, a.C, a.ncols, vo, a.col, a.st);
@@ -983,23 +1056,23 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     DevBuf srl, cl, cs, inv, src;
     if (Np > 0) {
         SELL_TRY(srl.alloc(al, Np * sizeof(int32_t), s));
-        SELL_TRY(cl.alloc(al, Nc * sizeof(int32_t), s));
+        SELL_TRY(cl.alloc(al, 2 * Nc * sizeof(int32_t), s));  // and the long rows per chunk
         SELL_TRY(src.alloc(al, Np * sizeof(int64_t), s));
-        SELL_CUDA_TRY(cudaMemsetAsync(cl.p, 0, Nc * sizeof(int32_t), s));
+        SELL_CUDA_TRY(cudaMemsetAsync(cl.p, 0, 2 * Nc * sizeof(int32_t), s));
     }
     const bool permute_cols = (o->flags & SELL_BUILD_PERMUTE_COLS) != 0;
     if (permute_cols && N > 0) SELL_TRY(inv.alloc(al, N * sizeof(int32_t), s));
     if (Np > 0) {
         int g = grid_for(Np, 256);
         k_chunk_len<<<g, 256, 0, s>>>(rl.as<int32_t>(), sorted ? perm.as<int32_t>() : nullptr, rpt, N, Np,
-                                      C, srl.as<int32_t>(), src.as<int64_t>(), cl.as<int32_t>(),
+                                      C, srl.as<int32_t>(), src.as<int64_t>(), cl.as<int32_t>(), cl.as<int32_t>() + Nc,
                                       permute_cols ? inv.as<int32_t>() : nullptr);
         SELL_CUDA_TRY(cudaGetLastError());
     }
     // 5. chunk offsets, and the chunks that hold rows longer than kSeg
     SELL_TRY(cs.alloc(al, (Nc + 1) * sizeof(int64_t), s));
-    DevBuf tile, lpos, ubase;
-    ChunkSums total = {0, 0, 0};
+    DevBuf tile, lpos, ubase, wbase;
+    ChunkSums total = {0, 0, 0, 0, 0};
     if (Nc > 0) {
         // tile sums, then the grand total; the block of tile t adds up the t
         // tile sums before it (at most 2048)
@@ -1008,11 +1081,14 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_TRY(tile.alloc(al, (nt + 1) * sizeof(ChunkSums), s));
         SELL_TRY(lpos.alloc(al, Nc * sizeof(int64_t), s));
         SELL_TRY(ubase.alloc(al, Nc * sizeof(int64_t), s));
+        SELL_TRY(wbase.alloc(al, Nc * sizeof(longlong2), s));
+        const int32_t *nlr = cl.as<int32_t>() + Nc;
         ChunkSums *tp = tile.as<ChunkSums>();
-        k_chunk_reduce<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), Nc, per, C, tp);
+        k_chunk_reduce<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), nlr, Nc, per, C, tp);
         SELL_CUDA_TRY(cudaGetLastError());
-        k_chunk_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), Nc, per, C, tp, cs.as<int64_t>(),
-                                                            lpos.as<int64_t>(), ubase.as<int64_t>(), tp + nt);
+        k_chunk_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), nlr, Nc, per, C, tp, cs.as<int64_t>(),
+                                                            lpos.as<int64_t>(), ubase.as<int64_t>(),
+                                                            wbase.as<longlong2>(), tp + nt);
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_CUDA_TRY(cudaMemcpyAsync(&total, tp + nt, sizeof(total), cudaMemcpyDeviceToHost, s));
         SELL_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1020,16 +1096,23 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_CUDA_TRY(cudaMemsetAsync(cs.p, 0, sizeof(int64_t), s));
     }
     const int64_t stored = total.stored, nlong = total.nlong, nunits = total.nunits;
-    DevBuf lchunk, lunit, cnt, cnt2, part, lrow, lmeta;
+    DevBuf lchunk, lunit, cnt, cnt2, part, lrow, lmeta, lwork, lval, lcol;
     if (nlong > 0) {
         SELL_TRY(lchunk.alloc(al, nlong * sizeof(int32_t), s));
         SELL_TRY(lunit.alloc(al, nunits * sizeof(int2), s));
         SELL_TRY(lrow.alloc(al, (size_t)nlong * C * sizeof(int32_t), s));
         SELL_TRY(lmeta.alloc(al, (size_t)nlong * sizeof(int4), s));
+        if (total.nwork > 0) SELL_TRY(lwork.alloc(al, (size_t)total.nwork * sizeof(LongWork), s));
+        if (total.npack > 0) {
+            SELL_TRY(lval.alloc(al, (size_t)total.npack * kSeg * 32 * value_size(o->store_type), s));
+            SELL_TRY(lcol.alloc(al, (size_t)total.npack * kSeg * 32 * sizeof(int32_t), s));
+        }
         k_long_lists<<<(unsigned)((Nc + 7) / 8), 256, 0, s>>>(cl.as<int32_t>(), srl.as<int32_t>(),
-                                                                  lpos.as<int64_t>(), ubase.as<int64_t>(), Nc, N, C,
+                                                                  lpos.as<int64_t>(), ubase.as<int64_t>(),
+                                                                  wbase.as<longlong2>(), cs.as<int64_t>(), Nc, N, C,
                                                                   lchunk.as<int32_t>(), lunit.as<int2>(),
-                                                                  lrow.as<int32_t>(), lmeta.as<int4>());
+                                                                  lrow.as<int32_t>(), lmeta.as<int4>(),
+                                                                  lwork.as<LongWork>());
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_TRY(cnt.alloc(al, nlong * C * sizeof(int32_t), s));
         SELL_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, nlong * C * sizeof(int32_t), s));
@@ -1056,7 +1139,12 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         a.cs = cs.as<int64_t>();
         a.lchunk = lchunk.as<int32_t>();
         a.lunit = lunit.as<int2>();
+        a.lrow = lrow.as<int32_t>();
+        a.lwork = lwork.as<LongWork>();
         a.nunits = nunits;
+        a.nlwork = total.nwork;
+        a.lval = lval.p;
+        a.lcol = lcol.as<int32_t>();
         a.N = N;
         a.Np = Np;
         a.ncols = A->ncols;
@@ -1079,12 +1167,12 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_CUDA_TRY(cudaStreamSynchronize(s));
         if (end.err) return malformed(end.err);
         // The products take the offsets where they save column bytes: at least
-        // half of the stored elements in slices with a pattern.  (Rows of one
+        // half of the entries in slices with a pattern.  (Rows of one
         // entry have a trivial one; a slice without one reads its columns.)
         unsigned long long nopat = 0;
         for (unsigned long long n : end.nopat) nopat += n;
         // The kernel loads offsets and prefetches values in 16-byte units.
-        pattern = tiled && 2 * nopat <= (unsigned long long)stored &&
+        pattern = tiled && 2 * nopat <= (unsigned long long)nnz &&
                   ((uintptr_t)val.p | (uintptr_t)scol.p) % 16 == 0;
     }
     if (!pattern) {
@@ -1115,10 +1203,14 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     h->al = al;
     h->nlong = nlong;
     h->nunits = nunits;
+    h->nlwork = total.nwork;
     h->part_k = nunits > 0 ? 1 : 0;
     h->device_bytes = val.bytes + col.bytes + cs.bytes + cl.bytes + srl.bytes + perm.bytes + lchunk.bytes +
                       lunit.bytes + cnt.bytes + cnt2.bytes + part.bytes + lrow.bytes + lmeta.bytes +
-                      scol.bytes + sflag.bytes;
+                      scol.bytes + sflag.bytes + lwork.bytes + lval.bytes + lcol.bytes;
+    h->lwork = (LongWork *)lwork.release_ownership();
+    h->lval = lval.release_ownership();
+    h->lcol = (int32_t *)lcol.release_ownership();
     h->scol = (int32_t *)scol.release_ownership();
     h->sflag = (int32_t *)sflag.release_ownership();
     h->lchunk = (int32_t *)lchunk.release_ownership();

@@ -25,6 +25,17 @@ __host__ __device__ __forceinline__ int64_t offset_start(int64_t cs0, int32_t wi
     return ((cs0 >> 5) + (int64_t)s * width + 3 * slice + 3) & ~(int64_t)3;
 }
 
+// A virtual warp of the long rows (sell_long.cuh): long chunk lc = chunk c,
+// whose first partial slot is u0 and which has nseg segments per row.
+// m < 0: segment i / (C / 32) of 32 neighbouring rows; else the 32 segments
+// from number 32 i of the chunk's m long rows, one row after another.  base:
+// where lane 0's first entry is.
+struct __align__(16) LongWork {
+    int32_t lc, c, nseg, m;
+    int64_t base;
+    int32_t i, u0;
+};
+
 // --------------------------------------------------------- device helpers
 // Streaming loads for data touched once per product (val/col): do not allocate
 // in L1 and mark the L2 lines evict-first, so that the gathered vector x keeps

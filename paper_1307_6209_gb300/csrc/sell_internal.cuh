@@ -120,6 +120,11 @@ struct sell_matrix {
     int32_t *lrow = nullptr;   // nlong * C lanes of each long chunk's long rows
     int4 *lmeta = nullptr;     // nlong {long rows, mode, units, 0} (sell_build.cu k_long_rows)
     int64_t nunits = 0;
+    // long rows of single products (sell_long.cuh; null when C is no multiple of 32)
+    sell::LongWork *lwork = nullptr;  // nlwork virtual warps
+    int64_t nlwork = 0;
+    void *lval = nullptr;      // entries of the virtual warps of chunks with few long rows,
+    int32_t *lcol = nullptr;   //   nlpack * kSeg * 32 of each
     int32_t *cnt = nullptr;    // nlong * C per-row segment counters (zero at rest)
     int32_t *cnt2 = nullptr;   // nunits * C group counters of very long rows (zero at rest)
     void *part = nullptr;      // segment partials: nunits * C * part_k * 8 bytes

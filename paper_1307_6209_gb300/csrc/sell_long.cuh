@@ -1,0 +1,289 @@
+// sell_long.cuh -- the rows longer than kSeg of a single product, in a kernel
+// of their own that runs ahead of the short rows' (sell_spmv_impl.cuh).
+//
+// Work: lwork lists the virtual warps (LongWork).  In a chunk of mostly long
+// rows (mode 0) a virtual warp takes one segment of 32 neighbouring rows; in
+// a chunk with few long rows (mode 1) it takes 32 consecutive segments of one
+// long row after another -- only as many virtual warps as there are segments.
+// The chunk holds such a row with a stride of C entries, one useful entry per
+// 32-byte sector; its virtual warps therefore have a copy of their entries,
+// entry j of lane t at base + j * 32 + t (lval, lcol: at most an eighth of the
+// chunk they come from), so that they read like a chunk of 32 full rows.
+// Chunk heights that are not a multiple of 32 go through the units of
+// sell_rowdot.cuh instead (lwork is null).
+//
+// Why a kernel of its own: with both paths in one kernel the long rows' fold
+// and loads set the registers of the short rows as well (binary64, one
+// vector: 56 against 32, i.e. 32 against 64 warps per SM).  The short rows'
+// kernel is launched behind this one as a programmatic dependent: its blocks
+// start as soon as every block of this kernel has started, so the two share
+// the chip, long rows first, and one thread of it waits for this kernel's end
+// before the whole product counts as finished.
+//
+// Every segment is the chain defined in sell_rowdot.cuh and the partials are
+// folded in segment order, so the results are the same bits.
+//
+// Bounds and measurements (binary64, one vector, block 128, against the long
+// rows in the first blocks of the short rows' launch): 10^6 rows of 3 and one
+// of 10^6 entries 70 -> 38 us (the row alone 29 us: 8 round trips of loads,
+// then chains of 256 and 62 dependent additions at 64 cycles each, the FP64
+// pipe's time for a warp); 500,000 lognormal rows unsorted 151 -> 112 us;
+// dense 8000^2 147 -> 127 us (FP64 pipe 104 us); 2M lognormal rows sorted
+// 133 -> 131 us (gathers).  Tried and slower: a block per 16 segments with
+// its entries in shared memory (200,000 sorted rows 26 -> 52 us, dense 402
+// us); 16 loads in flight (dense 144 us); prefetches of the packed entries
+// (500,000 unsorted rows 132 us).
+#pragma once
+
+#include "sell_rowdot.cuh"
+
+namespace sell {
+
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+constexpr int kLongThreads = 128;
+
+// The arrays of a matrix that the long rows need.
+struct LongArgs {
+    const int32_t *col;
+    const int64_t *cs;
+    const int32_t *srl, *perm, *lchunk, *lrow;
+    const int2 *lunit;
+    const int4 *lmeta;
+    const LongWork *lwork;
+    const int32_t *lcol;
+    Pattern pt;
+    int64_t nwork;  // virtual warps (lwork), or units (lunit) without lwork
+    int64_t N;
+    int C;
+};
+
+// One segment of a long row: long chunk lc, lane l of it, segment s of nseg;
+// its entry j is at base + j * stride of val / col, or of lval / lcol.
+struct LongSeg {
+    int64_t c, r, u0, base;  // chunk, sorted row, the chunk's first partial slot
+    int lc, l, s, nseg, L, stride;
+    bool valid, packed;
+};
+
+__device__ __forceinline__ void finish_segment(const LongArgs &a, LongSeg &g, bool in) {
+    g.r = g.c * a.C + g.l;
+    g.L = in && g.r < a.N ? a.srl[g.r] : 0;
+    g.nseg = (g.L - 1) / kSeg + 1;
+    g.valid = g.L > kSeg && g.s < g.nseg;
+}
+
+// Lane t of virtual warp w.
+__device__ __forceinline__ LongSeg long_segment(const LongArgs &a, int64_t w, int t) {
+    LongSeg g;
+    const LongWork wk = a.lwork[w];
+    g.lc = wk.lc;
+    g.c = wk.c;
+    g.u0 = wk.u0;
+    g.base = wk.base + t;
+    bool in = true;
+    if (wk.m < 0) {
+        const int spc = a.C >> 5;
+        g.s = wk.i / spc;
+        g.l = (wk.i - g.s * spc) * 32 + t;
+        g.stride = a.C;
+    } else {
+        const int64_t i = (int64_t)wk.i * 32 + t;
+        const int64_t k = i / wk.nseg;
+        in = k < wk.m;
+        g.s = (int)(i - k * wk.nseg);
+        g.l = in ? a.lrow[(int64_t)wk.lc * a.C + k] : 0;
+        g.stride = 32;
+    }
+    g.packed = wk.m >= 0;
+    finish_segment(a, g, in);
+    return g;
+}
+
+// Unit-thread v (chunk heights that are no multiple of 32).
+__device__ __forceinline__ LongSeg unit_segment(const LongArgs &a, int64_t v) {
+    LongSeg g;
+    const int64_t u = v / a.C;
+    const int t = (int)(v - u * a.C);
+    if (u >= a.nwork) return LongSeg{};
+    const int2 us = a.lunit[u];
+    const int4 meta = a.lmeta[us.x];
+    bool in = true;
+    g.lc = us.x;
+    g.u0 = u - us.y;
+    g.c = a.lchunk[us.x];
+    if (meta.y == 0) {
+        g.l = t;
+        g.s = us.y;
+    } else {
+        const int64_t i = (int64_t)us.y * a.C + t;  // beyond 32 bits for rows of more than 2^31 / C segments
+        const int64_t k = i / meta.z;
+        in = k < meta.x;
+        g.s = (int)(i - k * meta.z);
+        g.l = in ? a.lrow[(int64_t)us.x * a.C + k] : 0;
+    }
+    g.base = a.cs[g.c] + (int64_t)g.s * kSeg * a.C + g.l;
+    g.stride = a.C;
+    g.packed = false;
+    finish_segment(a, g, in);
+    return g;
+}
+
+__device__ __forceinline__ Plain<double> shfl_acc(const Plain<double> &v, int from) {
+    Plain<double> r;
+    r.s = __shfl_sync(0xffffffffu, v.s, from);
+    return r;
+}
+__device__ __forceinline__ Dot2 shfl_acc(const Dot2 &v, int from) {
+    Dot2 r;
+    r.p = __shfl_sync(0xffffffffu, v.p, from);
+    r.e = __shfl_sync(0xffffffffu, v.e, from);
+    return r;
+}
+
+// Folds, for the lanes with `done`, `count` partials each (as fold_partials).
+// Many lanes at once (a chunk of rows of one length completes together) fold
+// their own; few are folded one by one with the whole warp's loads, 32
+// partials in one round trip instead of a few: a group of 256 takes one trip
+// to L2 instead of 16.  All 32 lanes call.
+template <int K, class PT>
+__device__ __forceinline__ void fold_warp(bool done, const PT *part, int64_t base, int64_t stride, int count, int C,
+                                          int l, PT (&tot)[K]) {
+    const int lane = threadIdx.x & 31;
+    unsigned todo = __ballot_sync(0xffffffffu, done);
+    if (__popc(todo) > 4) {
+        if (done) fold_partials<K, PT>(part, base, stride, count, C, l, tot);
+        __syncwarp();
+        return;
+    }
+    __syncwarp();  // the owner's fence holds for the loads of the other lanes
+    constexpr int Q = K == 1 ? 8 : 1;  // rounds of 32 loads in flight
+    for (; todo; todo &= todo - 1) {
+        const int owner = __ffs(todo) - 1;
+        const int64_t b = __shfl_sync(0xffffffffu, base, owner);
+        const int n = __shfl_sync(0xffffffffu, count, owner), ll = __shfl_sync(0xffffffffu, l, owner);
+        PT sum[K];
+        for (int i0 = 0; i0 < n; i0 += 32 * Q) {
+            PT p[Q][K];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int i = i0 + q * 32 + lane;
+                if (i < n) {
+#pragma unroll
+                    for (int e = 0; e < K; ++e) p[q][e] = PT::load_l2(part + ((b + i * stride) * C + ll) * K + e);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int m = min(32, n - i0 - q * 32);
+                for (int t = 0; t < m; ++t) {
+#pragma unroll
+                    for (int e = 0; e < K; ++e) {
+                        const PT v = shfl_acc(p[q][e], t);
+                        if (i0 + q * 32 + t == 0) sum[e] = v;
+                        else sum[e].merge(v);
+                    }
+                }
+            }
+        }
+        if (lane == owner) {
+#pragma unroll
+            for (int e = 0; e < K; ++e) tot[e] = sum[e];
+        }
+    }
+}
+
+// Stores the segments' partials and folds the rows (or groups) that they
+// complete.  All 32 lanes call; acc counts where g.valid.
+template <class XT, int K, class Acc>
+__device__ __forceinline__ void long_finish(const LongArgs &a, const LongSeg &g, const Acc (&acc)[K], void *part,
+                                            int32_t *cnt, int32_t *cnt2, XT *Y, int64_t ldy) {
+    using PT = typename PartOf<Acc>::T;
+    PT *pp = static_cast<PT *>(part);
+    const int C = a.C;
+    int32_t *ct = cnt + (int64_t)g.lc * C + g.l;
+    bool done = false;
+    const bool big = g.valid && g.nseg > kSuper;
+    if (g.valid) {
+#pragma unroll
+        for (int q = 0; q < K; ++q) pp[((g.u0 + g.s) * C + g.l) * K + q] = PartOf<Acc>::from(acc[q]);
+    }
+    const int s0 = (g.s / kSuper) * kSuper, ng = min(kSuper, g.nseg - s0);
+    PT tot[K];
+    if (__any_sync(0xffffffffu, big)) {
+        int32_t *cg = cnt2 + (g.u0 + s0) * C + g.l;
+        bool last = false;  // this lane completed its group
+        if (big) {
+            __threadfence();
+            last = atomicAdd(cg, 1) == ng - 1;
+            if (last) __threadfence();
+        }
+        fold_warp<K, PT>(last, pp, g.u0 + s0, 1, ng, C, g.l, tot);
+        if (last) {
+            *cg = 0;
+#pragma unroll
+            for (int q = 0; q < K; ++q) pp[((g.u0 + s0) * C + g.l) * K + q] = tot[q];
+            __threadfence();
+            done = atomicAdd(ct, 1) == (g.nseg + kSuper - 1) / kSuper - 1;
+        }
+    }
+    if (g.valid && !big) {
+        __threadfence();
+        done = atomicAdd(ct, 1) == g.nseg - 1;
+    }
+    if (done) __threadfence();
+    // rows of up to kSuper segments fold those, the others their groups
+    const unsigned bigs = __ballot_sync(0xffffffffu, done && big);
+    if (bigs) fold_warp<K, PT>(done && big, pp, g.u0, kSuper, (g.nseg + kSuper - 1) / kSuper, C, g.l, tot);
+    if (__any_sync(0xffffffffu, done && !big)) fold_warp<K, PT>(done && !big, pp, g.u0, 1, g.nseg, C, g.l, tot);
+    if (done) {
+        const int64_t out = a.perm ? (int64_t)a.perm[g.r] : g.r;
+#pragma unroll
+        for (int q = 0; q < K; ++q) Y[out * ldy + q] = static_cast<XT>(tot[q].result());
+        *ct = 0;
+    }
+}
+
+template <class VT, int K, int U, bool PIPE, class Acc, bool PAT>
+__global__ void __launch_bounds__(kLongThreads)
+k_long(const VT *__restrict__ val, const VT *__restrict__ lval, const LongArgs a, void *part, int32_t *cnt,
+       int32_t *cnt2, const typename XType<VT>::T *__restrict__ X, int64_t ldx, typename XType<VT>::T *Y,
+       int64_t ldy, int accumulate, int vec) {
+    using XT = typename XType<VT>::T;
+    dependents_may_start();
+    const int64_t v = blockIdx.x * (int64_t)kLongThreads + threadIdx.x;
+    LongSeg g;
+    if (a.lwork) {
+        if (v / 32 >= a.nwork) return;
+        g = long_segment(a, v / 32, threadIdx.x & 31);
+    } else {
+        g = unit_segment(a, v);
+    }
+    const uint64_t pol = l2_evict_first_policy();
+    Acc acc[K];
+    if (g.valid) {
+        const int64_t out = a.perm ? (int64_t)a.perm[g.r] : g.r;
+#pragma unroll
+        for (int q = 0; q < K; ++q) acc[q].init((g.s == 0 && accumulate) ? Y[out * ldy + q] : XT(0));
+        const int n = min(g.L - g.s * kSeg, kSeg);
+        const VT *vp = (g.packed ? lval : val) + g.base;
+        bool done = false;
+        if constexpr (PAT) {
+            if (!g.packed && a.pt.flag[g.r >> 5]) {
+                const int64_t cs0 = a.cs[g.c];
+                const int32_t *op = a.pt.off + offset_start(cs0, a.pt.cl[g.c], g.l >> 5, g.r >> 5) + g.s * kSeg;
+                chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, vp, op, __ldg(a.col + cs0 + g.l), g.stride, 0, n, X,
+                                                          ldx, vec & 3, pol);
+                done = true;
+            }
+        }
+        if (!done)
+            chain<VT, XT, K, U, PIPE, Acc>(acc, vp, (g.packed ? a.lcol : a.col) + g.base, g.stride, 0, n, X, ldx,
+                                           vec & 3, pol);
+    }
+    __syncwarp();
+    long_finish<XT, K, Acc>(a, g, acc, part, cnt, cnt2, Y, ldy);
+}
+
+}  // namespace sell

@@ -521,7 +521,8 @@ __device__ __forceinline__ void fold_partials(const Acc *part, int64_t base, int
     }
 }
 
-// One thread of a long-row work unit.  Units are (long chunk lc, segment s)
+// One thread of a long-row work unit (batches and the bulk-staged kernel; the
+// single products' long rows are in sell_long.cuh).  Units are (long chunk lc, segment s)
 // pairs, numbered chunk by chunk (lunit[u] = {lc, s}); a unit has C threads,
 // virtual thread v = u*C + l takes lane l.  part holds K Accs per (unit,
 // lane); cnt one counter per (long chunk, lane) and cnt2 one per (unit,
@@ -533,13 +534,10 @@ __device__ __forceinline__ void fold_partials(const Acc *part, int64_t base, int
 // that completes the group (its result replaces the group's first partial),
 // then the thread that completes the last group folds the group results in
 // order.  Either way the result depends only on the row's entries.
-//
-// PAT: the matrix has slices with one column pattern (pt; C is a multiple of
-// 32).
-template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT = false>
+template <class VT, class XT, int K, int U, bool PIPE, class Acc>
 __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const int32_t *__restrict__ srl,
-                                          const int32_t *__restrict__ perm, const Pattern &pt, const int32_t *__restrict__ lchunk,
+                                          const int32_t *__restrict__ perm, const int32_t *__restrict__ lchunk,
                                           const int2 *__restrict__ lunit, const int4 *__restrict__ lmeta,
                                           const int32_t *__restrict__ lrow, Acc *part, int32_t *cnt,
                                           int32_t *cnt2, const XT *__restrict__ X, int64_t ldx, XT *Y,
@@ -572,8 +570,9 @@ __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int3
     Acc acc[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) acc[q].init((s == 0 && accumulate) ? Y[out * ldy + q] : XT(0));
-    row_chain<VT, XT, K, U, PIPE, Acc, PAT>(acc, val, col, cs, pt, C, r, c, l, s * kSeg, min(L, (s + 1) * kSeg), X,
-                                            ldx, vec & 3, pol);
+    const int64_t base = cs[c] + l;
+    chain<VT, XT, K, U, PIPE, Acc>(acc, val + base, col + base, C, s * kSeg, min(L, (s + 1) * kSeg), X, ldx,
+                                   vec & 3, pol);
     using PT = typename PartOf<Acc>::T;
     PT *pp = reinterpret_cast<PT *>(part);
 #pragma unroll

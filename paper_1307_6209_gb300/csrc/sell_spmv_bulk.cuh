@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(512) k_spmv_bulk(const __grid_constant__ Args<
     // ---- long-row work units first (their copies above are already in flight)
     if constexpr (LONG) {
         for (int64_t v = wg * 32 + lane; v < a.long_threads; v += NW * 32)
-            long_unit<VT, XT, 1, 4, false, Acc>(a.val, a.col, a.cs, a.srl, a.perm, Pattern{}, a.lchunk, a.lunit, a.lmeta,
+            long_unit<VT, XT, 1, 4, false, Acc>(a.val, a.col, a.cs, a.srl, a.perm, a.lchunk, a.lunit, a.lmeta,
                                                 a.lrow, a.part, a.cnt, a.cnt2, a.X, a.ldx, a.Y, a.ldy, a.N, C, v,
                                                 a.accumulate, false, pol);
         __syncwarp();
