@@ -253,6 +253,8 @@ SELL_API sell_status sell_spmmv_noalloc(sell_handle h, const void *X, int64_t ld
  * results do not depend on any of these settings.  (A handle most of whose
  * 32-row slices have one column pattern -- structured grids, dense blocks --
  * uses kernels of its own in modes 0 and 1, which take only the block.)
+ * What was never set is the library's choice by value type and number of
+ * right-hand sides (block 128, pipelined).
  *   block    threads per block (32..512, multiple of 32); 0 keeps it.
  *   unroll   entries of a row loaded per step (1, 2, 4 or 8); 0 keeps it.
  *   pipeline how the matrix stream (val/col) is read; -1 keeps it:

@@ -92,8 +92,9 @@ sell_status bulk_prepare(sell_matrix *h) {
     // bulk copies need 16-byte aligned sources (chunk offsets are multiples of C)
     if (((uintptr_t)h->val | (uintptr_t)h->col | (uintptr_t)h->srl) % 16 != 0)
         return fail(SELL_EUNSUPPORTED, "bulk-staged SpMV needs 16-byte aligned format arrays");
-    const int W = h->block / 32;
-    int R = h->unroll >= 8 ? 4 : (h->unroll >= 4 ? 3 : (h->unroll >= 2 ? 2 : 1));
+    const int W = (h->block ? h->block : 256) / 32;
+    const int u = h->unroll ? h->unroll : 4;
+    int R = u >= 8 ? 4 : (u >= 4 ? 3 : (u >= 2 ? 2 : 1));
     int bps = 0;
     for (; R >= 1; --R) {
         switch (h->store_type) {

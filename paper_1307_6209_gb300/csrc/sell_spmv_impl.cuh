@@ -110,6 +110,12 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
     return cudaGetLastError();
 }
 
+// Threads per block unless sell_set_launch says otherwise: a block's warps
+// leave the SM together, so the small ones lose less to rows of different
+// lengths (2M sorted lognormal rows binary64, unroll 4: block 128 132.7 us,
+// 256 137.4 us, 512 141.7 us; 64 gains nothing more).
+constexpr int kBlock = 128;
+
 // One launch of a short-row kernel, behind the long rows' where there are any.
 template <class VT, class Kernel>
 cudaError_t launch_short(Kernel kern, const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc,
@@ -120,15 +126,16 @@ cudaError_t launch_short(Kernel kern, const sell_matrix *h, const void *X, int64
     const XT *x = static_cast<const XT *>(X);
     XT *y = static_cast<XT *>(Y);
     const Pattern pt{h->scol, h->sflag, h->cl};
-    const unsigned blocks = (unsigned)((h->nrows + h->block - 1) / h->block);
+    const int block = h->block ? h->block : kBlock;
+    const unsigned blocks = (unsigned)((h->nrows + block - 1) / block);
     if (!h->nunits) {
-        kern<<<blocks, h->block, 0, s>>>(val, h->col, h->cs, h->srl, perm, pt, x, ldx, y, ldy, h->nrows, h->C, acc, vec,
+        kern<<<blocks, block, 0, s>>>(val, h->col, h->cs, h->srl, perm, pt, x, ldx, y, ldy, h->nrows, h->C, acc, vec,
                                          0);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks + 1);
-    cfg.blockDim = dim3(h->block);
+    cfg.blockDim = dim3(block);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -175,7 +182,7 @@ cudaError_t run_pattern(const sell_matrix *h, const void *X, int64_t ldx, void *
 template <class VT, int K, bool PIPE, class Acc>
 cudaError_t pick_u(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc, int vec,
                    cudaStream_t s) {
-    int u = h->unroll;
+    const int u = h->unroll ? h->unroll : 4;
     if constexpr (K >= 8) {
         return u >= 2 ? run<VT, K, 2, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s)
                       : run<VT, K, 1, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
@@ -192,7 +199,15 @@ cudaError_t pick_u(const sell_matrix *h, const void *X, int64_t ldx, void *Y, in
 }
 
 // K columns: the long rows, then the short ones.  Launch mode 1 runs the
-// software-pipelined chain at every block width.
+// software-pipelined chain at every block width.  Without sell_set_launch the
+// chain is pipelined, with the unroll that was fastest or within 4 % of it on
+// the matrices it was swept on (block 128; unroll 4 without pipelining, block
+// 256 in brackets): binary64 at one vector unroll 2: 1M banded rows 66.9 us
+// [92.2], 2M sorted lognormal rows 133 us [137]; binary32 at one vector unroll
+// 4: 1M banded rows 33.2 us [36.8]; four vectors 4 (binary64 2): 1M lognormal
+// rows binary32 98 us [131], 1M banded rows binary64 149 us [187]; eight
+// vectors 2 (binary64 1): 1M lognormal rows binary32 105 us [117], binary64
+// 219 us [269], 1M banded rows binary32 77 us [103].
 template <class VT, int K, class Acc, class AccL>
 cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc, int vec,
                       void *part, int32_t *cnt, int32_t *cnt2, cudaStream_t s) {
@@ -202,7 +217,12 @@ cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
     }
     if (h->scol && ldx < (1 << 28))  // row pitches beyond 2^31 bytes keep the general kernels
         return run_pattern<VT, K, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
-    if (h->pipeline == 1) return pick_u<VT, K, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+    // (launch mode 2 is the bulk-staged kernel's: its unroll counts slots)
+    if ((h->pipeline != 0 && h->unroll == 0) || h->pipeline == 2) {
+        constexpr int U = K == 8 ? 2 : 4;
+        return run<VT, K, sizeof(VT) == 8 ? U / 2 : U, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+    }
+    if (h->pipeline != 0) return pick_u<VT, K, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     return pick_u<VT, K, false, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
 }
 
