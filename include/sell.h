@@ -326,12 +326,14 @@ typedef struct {
 
 typedef struct sell_batch *sell_batch_plan;
 
-/* Prepare a batch of n products to run in a few launches (one per kernel
- * variant present -- value type, block of 1/2/4/8 right-hand sides, plain or
- * compensated accumulation -- and per 160 products).  Work units are tiles of
+/* Prepare a batch of n products to run in a few launches (per kernel variant
+ * present -- value type, block of 1/2/4/8 right-hand sides, plain or
+ * compensated accumulation -- and per 144 products, one for the long rows and
+ * one for the others).  Work units are tiles of
  * 128 sorted rows of one product, or 128 threads of its long-row segment
  * work (sell_batch_set_launch changes the size); every launch has one block
- * per unit, long-row work first and the biggest products first.  The
+ * per unit, the biggest products first, the long rows' launches before the
+ * others.  The
  * products may use matrices of different sizes and storage types; a matrix
  * with more than 8 right-hand sides is split into blocks of 8 (or of the
  * item's SELL_SPMV_RHS_BLOCK* width).  Each result is bit-identical to the same product run

@@ -82,6 +82,10 @@ inline int rhs_block(int rem, int maxw) {
     return kb;
 }
 
+// Row pitches of X from here on (in elements) take 64-bit arithmetic: one
+// column at a time, in kernels of their own (sell_rowdot.cuh, WidePitch).
+constexpr int64_t kWidePitch = 1 << 28;
+
 // How the kernels may load a row of X, or store a row of Y (base, row pitch
 // ld elements of xs bytes): 2 with 32-byte vectors, 1 with 16-byte vectors,
 // 0 value by value.  The kernels take X's in bits 0-1 and Y's in bits 2-3.
@@ -163,6 +167,7 @@ struct sell_batch {
     struct Group {              // one launch: kernel variant, its products and units
         void *fn = nullptr;     // kernel entry
         void *params = nullptr; // host copy of the launch parameters (products and their unit ranges)
+        bool lng = false;       // long rows (else short rows)
         int64_t nwork = 0;
         int32_t grid = 0;
     };

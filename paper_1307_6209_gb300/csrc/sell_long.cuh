@@ -245,14 +245,14 @@ __device__ __forceinline__ void long_finish(const LongArgs &a, const LongSeg &g,
     }
 }
 
-template <class VT, int K, int U, bool PIPE, class Acc, bool PAT>
-__global__ void __launch_bounds__(kLongThreads)
-k_long(const VT *__restrict__ val, const VT *__restrict__ lval, const LongArgs a, void *part, int32_t *cnt,
-       int32_t *cnt2, const typename XType<VT>::T *__restrict__ X, int64_t ldx, typename XType<VT>::T *Y,
-       int64_t ldy, int accumulate, int vec) {
+// Thread v of a product's long-row work (v / 32 = virtual warp; all 32 lanes
+// of a warp call together, with blocks of a multiple of 32 threads).
+template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, class LD>
+__device__ __forceinline__ void long_rows(const VT *__restrict__ val, const VT *__restrict__ lval, const LongArgs &a,
+                                          void *part, int32_t *cnt, int32_t *cnt2,
+                                          const typename XType<VT>::T *__restrict__ X, LD ldx,
+                                          typename XType<VT>::T *Y, int64_t ldy, int accumulate, int vec, int64_t v) {
     using XT = typename XType<VT>::T;
-    dependents_may_start();
-    const int64_t v = blockIdx.x * (int64_t)kLongThreads + threadIdx.x;
     LongSeg g;
     if (a.lwork) {
         if (v / 32 >= a.nwork) return;
@@ -285,5 +285,37 @@ k_long(const VT *__restrict__ val, const VT *__restrict__ lval, const LongArgs a
     __syncwarp();
     long_finish<XT, K, Acc>(a, g, acc, part, cnt, cnt2, Y, ldy);
 }
+
+template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, class LD>
+__global__ void __launch_bounds__(kLongThreads)
+k_long(const VT *__restrict__ val, const VT *__restrict__ lval, const LongArgs a, void *part, int32_t *cnt,
+       int32_t *cnt2, const typename XType<VT>::T *__restrict__ X, LD ldx, typename XType<VT>::T *Y,
+       int64_t ldy, int accumulate, int vec) {
+    dependents_may_start();
+    long_rows<VT, K, U, PIPE, Acc, PAT>(val, lval, a, part, cnt, cnt2, X, ldx, Y, ldy, accumulate, vec,
+                                        blockIdx.x * (int64_t)kLongThreads + threadIdx.x);
+}
+
+// The long-row arguments of a handle (with its column patterns or not).
+inline LongArgs long_args(const sell_matrix *h, bool pattern) {
+    LongArgs a;
+    a.col = h->col;
+    a.cs = h->cs;
+    a.srl = h->srl;
+    a.perm = (h->flags & SELL_BUILD_PERMUTE_COLS) ? nullptr : h->perm;
+    a.lchunk = h->lchunk;
+    a.lrow = h->lrow;
+    a.lunit = h->lunit;
+    a.lmeta = h->lmeta;
+    a.lwork = h->lwork;
+    a.lcol = h->lcol;
+    a.pt = pattern ? Pattern{h->scol, h->sflag, h->cl} : Pattern{};
+    a.nwork = h->lwork ? h->nlwork : h->nunits;
+    a.N = h->nrows;
+    a.C = h->C;
+    return a;
+}
+// Its threads.
+inline int64_t long_threads(const sell_matrix *h) { return h->lwork ? h->nlwork * 32 : h->nunits * h->C; }
 
 }  // namespace sell

@@ -69,7 +69,7 @@ extern "C" sell_status sell_spmmv_noalloc(sell_handle h, const void *X, int64_t 
     const size_t cnt2_bytes = ((size_t)h->nunits * h->C * sizeof(int32_t) + 255) / 256 * 256;
     const size_t cnt_bytes = cnt1_bytes + cnt2_bytes;
     const size_t per_col = (size_t)h->nunits * h->C * 8;
-    int kmax = 8;
+    int kmax = ldx < kWidePitch ? 8 : 1;
     while (kmax > 1 && cnt_bytes + per_col * kmax > kScratchBytes) kmax >>= 1;
     if (cnt_bytes + per_col * kmax > kScratchBytes)
         return fail(SELL_EINVAL, "sell_spmmv_noalloc: the matrix's long rows need " +

@@ -165,9 +165,29 @@ __device__ __forceinline__ void load_x_at(const XT *__restrict__ p, int vec, XT 
     }
 }
 
-template <int K, class XT>
-__device__ __forceinline__ void load_x(const XT *__restrict__ X, int64_t ldx, int32_t ci, int vec, XT (&xv)[K]) {
-    load_x_at<K>(X + (int64_t)ci * ldx, vec, xv);
+// The row pitch of X: in bytes, where that fits 31 bits (a row's address is
+// then one multiply-add and the pitch one register), else in elements.
+struct Pitch {
+    int32_t bytes;
+};
+using WidePitch = int64_t;
+template <class XT>
+__device__ __forceinline__ const XT *x_row(const XT *X, Pitch p, int32_t ci) {
+    return reinterpret_cast<const XT *>(reinterpret_cast<const char *>(X) + (int64_t)ci * p.bytes);
+}
+template <class XT>
+__device__ __forceinline__ const XT *x_row(const XT *X, WidePitch ldx, int32_t ci) {
+    return X + (int64_t)ci * ldx;
+}
+template <int K, class XT, class LD>
+__device__ __forceinline__ void load_x(const XT *__restrict__ X, LD ldx, int32_t ci, int vec, XT (&xv)[K]) {
+    load_x_at<K>(x_row(X, ldx, ci), vec, xv);
+}
+
+// p + u * C elements, as one multiply-add of 32-bit factors (u is a constant).
+template <class T>
+__device__ __forceinline__ const T *column(const T *p, int C, int u) {
+    return reinterpret_cast<const T *>(reinterpret_cast<const char *>(p) + (int64_t)C * (u * (int)sizeof(T)));
 }
 
 // 32 bytes of Y at p (32-byte aligned) in one 256-bit store or load.
@@ -268,13 +288,13 @@ __device__ __forceinline__ void load_y(const XT *Y, int64_t ldy, int64_t i, int 
 // PIPE the stream loads of the next group are issued before the gathers and
 // FMAs of the current one (software pipelining: more bytes in flight per
 // thread; the order of the FMAs is unchanged).
-template <class VT, class XT, int K, int U, bool PIPE, class Acc>
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, int CT = 0, class LD>
 __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
-                                      const int32_t *__restrict__ cp, int C, int j0, int j1,
-                                      const XT *__restrict__ X, int64_t ldx, int vec, uint64_t pol) {
-    const int64_t stride = C;
-    vp += (int64_t)j0 * stride;
-    cp += (int64_t)j0 * stride;
+                                      const int32_t *__restrict__ cp, int height, int j0, int j1,
+                                      const XT *__restrict__ X, LD ldx, int vec, uint64_t pol) {
+    const int C = CT ? CT : height;
+    vp += (int64_t)j0 * C;
+    cp += (int64_t)j0 * C;
     int j = j0;
     if constexpr (PIPE) {
         if (j + U <= j1) {
@@ -282,8 +302,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
             int32_t ci[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                v[u] = ld_stream(vp + u * stride, pol);
-                ci[u] = ld_stream(cp + u * stride, pol);
+                v[u] = ld_stream(column(vp, C, u), pol);
+                ci[u] = ld_stream(column(cp, C, u), pol);
             }
             for (;;) {
                 const bool more = j + 2 * U <= j1;
@@ -292,8 +312,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
                 if (more) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        vn[u] = ld_stream(vp + (U + u) * stride, pol);
-                        cn[u] = ld_stream(cp + (U + u) * stride, pol);
+                        vn[u] = ld_stream(column(vp, C, U + u), pol);
+                        cn[u] = ld_stream(column(cp, C, U + u), pol);
                     }
                 }
                 XT xv[U][K];
@@ -305,8 +325,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
 #pragma unroll
                     for (int q = 0; q < K; ++q) acc[q].add(a, xv[u][q]);
                 }
-                vp += U * stride;
-                cp += U * stride;
+                vp = column(vp, C, U);
+                cp = column(cp, C, U);
                 j += U;
                 if (!more) break;
 #pragma unroll
@@ -322,8 +342,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
             int32_t ci[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                v[u] = ld_stream(vp + u * stride, pol);
-                ci[u] = ld_stream(cp + u * stride, pol);
+                v[u] = ld_stream(column(vp, C, u), pol);
+                ci[u] = ld_stream(column(cp, C, u), pol);
             }
             XT xv[U][K];
 #pragma unroll
@@ -334,8 +354,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
 #pragma unroll
                 for (int q = 0; q < K; ++q) acc[q].add(a, xv[u][q]);
             }
-            vp += U * stride;
-            cp += U * stride;
+            vp = column(vp, C, U);
+            cp = column(cp, C, U);
         }
     }
     if constexpr (U > 1) {
@@ -345,8 +365,8 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
 #pragma unroll
             for (int u = 0; u < U - 1; ++u) {
                 if (j + u < j1) {
-                    v[u] = ld_stream(vp + u * stride, pol);
-                    ci[u] = ld_stream(cp + u * stride, pol);
+                    v[u] = ld_stream(column(vp, C, u), pol);
+                    ci[u] = ld_stream(column(cp, C, u), pol);
                 }
             }
             XT xv[U][K];
@@ -373,12 +393,9 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
 template <class VT, class XT, int K, int U, bool PIPE, int CT, class Acc>
 __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restrict__ vp,
                                               const int32_t *__restrict__ op, int32_t first, int C, int j0, int j1,
-                                              const XT *__restrict__ X, int64_t ldx, int vec, uint64_t pol) {
-    const int64_t stride = CT ? CT : C;
-    // the row pitch of X in bytes fits 31 bits (run_pattern), so that a row's
-    // address is one multiply-add
-    const char *xp = reinterpret_cast<const char *>(X + (int64_t)first * ldx);
-    const int32_t pitch = (int32_t)(ldx * (int64_t)sizeof(XT));
+                                              const XT *__restrict__ X, Pitch ldx, int vec, uint64_t pol) {
+    const int stride = CT ? CT : C;
+    const XT *xp = x_row(X, ldx, first);
     op += j0;
     vp += (int64_t)j0 * stride;
     constexpr int XB = K >= 8 && U > 2 ? 2 : U;  // rows of X in flight
@@ -390,7 +407,7 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
 #pragma unroll
             for (int u = 0; u < XB; ++u)
                 if (b + u < n)
-                    load_x_at<K>(reinterpret_cast<const XT *>(xp + (int64_t)o[b + u] * pitch), vec, xv[u]);
+                    load_x<K>(xp, ldx, o[b + u], vec, xv[u]);
 #pragma unroll
             for (int u = 0; u < XB; ++u) {
                 if (b + u < n) {
@@ -424,20 +441,20 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
             offsets(o, 0);
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u < j1) v[u] = ld_stream(vp + u * stride, pol);
+                if (j + u < j1) v[u] = ld_stream(column(vp, stride, u), pol);
         }
         for (; j + U < j1; j += U) {
             offsets(on, U);
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + U + u < j1) vn[u] = ld_stream(vp + (U + u) * stride, pol);
+                if (j + U + u < j1) vn[u] = ld_stream(column(vp, stride, U + u), pol);
             group(v, o, U);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 v[u] = vn[u];
                 o[u] = on[u];
             }
-            vp += U * stride;
+            vp = column(vp, stride, U);
             op += U;
         }
         if (j < j1) group(v, o, j1 - j);
@@ -447,9 +464,9 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
             int32_t o[U];
             offsets(o, 0);
 #pragma unroll
-            for (int u = 0; u < U; ++u) v[u] = ld_stream(vp + u * stride, pol);
+            for (int u = 0; u < U; ++u) v[u] = ld_stream(column(vp, stride, u), pol);
             group(v, o, U);
-            vp += U * stride;
+            vp = column(vp, stride, U);
             op += U;
         }
         if (j < j1) {
@@ -458,7 +475,7 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
             offsets(o, 0);
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u < j1) v[u] = ld_stream(vp + u * stride, pol);
+                if (j + u < j1) v[u] = ld_stream(column(vp, stride, u), pol);
             group(v, o, j1 - j);
         }
     }
@@ -466,10 +483,10 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
 
 // The chain over entries j0..j1-1 of sorted row r = lane l of chunk c.
 // PAT: the matrix has slices with one column pattern.
-template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT>
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT, int CT, class LD>
 __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const Pattern &pt, int C, int64_t r,
-                                          int64_t c, int l, int j0, int j1, const XT *__restrict__ X, int64_t ldx,
+                                          int64_t c, int l, int j0, int j1, const XT *__restrict__ X, LD ldx,
                                           int vec, uint64_t pol) {
     const int64_t cs0 = cs[c];
     const int64_t base = cs0 + l;
@@ -486,13 +503,18 @@ __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ 
             if (n <= 0) return;
             const int32_t first = __ldg(col + base);
             const int32_t *op = pt.off + offset_start(cs0, width, l >> 5, r >> 5);
-            if (C == 32) chain_pattern<VT, XT, K, U, PIPE, 32, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
-            else chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+            if constexpr (sizeof(XT) == 4) {  // binary64 waits for the FP64 pipe, not for its addresses
+                if (C == 32) {
+                    chain_pattern<VT, XT, K, U, PIPE, 32, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+                    return;
+                }
+            }
+            chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
             return;
         }
         if (ask) prefetch_l2(col + at, (uint32_t)(n * 128), pol);
     }
-    chain<VT, XT, K, U, PIPE, Acc>(acc, val + base, col + base, C, j0, j1, X, ldx, vec, pol);
+    chain<VT, XT, K, U, PIPE, Acc, CT>(acc, val + base, col + base, C, j0, j1, X, ldx, vec, pol);
 }
 
 // Fold `count` partials of lane l, found at units base, base + stride, ...,
@@ -607,17 +629,18 @@ __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int3
 }
 
 // The thread's own row when it is short (L <= kSeg); long rows return.
-template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT = false>
+template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT = false, int CT = 0, class LD>
 __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const int32_t *__restrict__ srl,
                                           const int32_t *__restrict__ perm, const Pattern &pt, const XT *__restrict__ X,
-                                          int64_t ldx, XT *Y, int64_t ldy, int C, int64_t r, int accumulate,
+                                          LD ldx, XT *Y, int64_t ldy, int C, uint32_t r, int accumulate,
                                           int vec, uint64_t pol) {
     const int L = srl[r];
     if (L > kSeg) return;
-    const uint32_t c = (uint32_t)r / (uint32_t)C;  // padded row numbers stay below 2^31
-    const int l = (int)((uint32_t)r - c * (uint32_t)C);
-    const int64_t out = perm ? (int64_t)perm[r] : r;
+    const uint32_t height = CT ? CT : C;
+    const uint32_t c = r / height;  // padded row numbers stay below 2^31
+    const int l = (int)(r - c * height);
+    const uint32_t out = perm ? (uint32_t)perm[r] : r;
     Acc acc[K];
     if (accumulate) {
         XT y0[K];
@@ -628,7 +651,7 @@ __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int3
 #pragma unroll
         for (int q = 0; q < K; ++q) acc[q].init(XT(0));
     }
-    row_chain<VT, XT, K, U, PIPE, Acc, PAT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec & 3, pol);
+    row_chain<VT, XT, K, U, PIPE, Acc, PAT, CT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec & 3, pol);
     XT yo[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) yo[q] = acc[q].result();

@@ -39,7 +39,7 @@ cudaError_t dispatch(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
 sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy,
                          int32_t k, uint32_t flags, cudaStream_t s) {
     if (h->nrows == 0) return SELL_OK;
-    const int maxw = max_rhs_block(flags);
+    const int maxw = ldx < kWidePitch ? max_rhs_block(flags) : 1;
     if (h->nunits > 0) {
         const int need = rhs_block(k, maxw);
         if (need > h->part_k) {

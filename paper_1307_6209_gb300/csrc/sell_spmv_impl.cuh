@@ -31,7 +31,7 @@ namespace spmv_impl {
 #define SELL_SPMMV_PARAMS                                                                              \
     const VT *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ cs,      \
         const int32_t *__restrict__ srl, const int32_t *__restrict__ perm, const Pattern pt,          \
-        const typename XType<VT>::T *__restrict__ X, int64_t ldx, typename XType<VT>::T *Y, int64_t ldy, \
+        const typename XType<VT>::T *__restrict__ X, LD ldx, typename XType<VT>::T *Y, int64_t ldy,    \
         int64_t N, int C, int accumulate, int vec, int after_long
 #define SELL_SPMMV_ARGS val, col, cs, srl, perm, pt, X, ldx, Y, ldy, N, C, accumulate, vec, after_long
 
@@ -39,7 +39,7 @@ namespace spmv_impl {
 // rows' kernel (sell_long.cuh) runs ahead of this one, which ends only once
 // that has ended: the threads past the last row wait for it (launch_short
 // adds a block of them, so that there are some).
-template <class VT, int K, int U, bool PIPE, class Acc, bool PAT = false>
+template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, int CT, class LD>
 __device__ __forceinline__ void spmmv_body(SELL_SPMMV_PARAMS) {
     using XT = typename XType<VT>::T;
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -47,13 +47,13 @@ __device__ __forceinline__ void spmmv_body(SELL_SPMMV_PARAMS) {
         if (after_long) wait_for_predecessor();
         return;
     }
-    short_row<VT, XT, K, U, PIPE, Acc, PAT>(val, col, cs, srl, perm, pt, X, ldx, Y, ldy, C, r, accumulate, vec,
-                                            l2_evict_first_policy());
+    short_row<VT, XT, K, U, PIPE, Acc, PAT, CT>(val, col, cs, srl, perm, pt, X, ldx, Y, ldy, C, (uint32_t)r, accumulate,
+                                            vec, l2_evict_first_policy());
 }
 
-template <class VT, int K, int U, bool PIPE, class Acc>
+template <class VT, int K, int U, bool PIPE, class Acc, class LD = Pitch>
 __global__ void __launch_bounds__(512) k_spmmv(SELL_SPMMV_PARAMS) {
-    spmmv_body<VT, K, U, PIPE, Acc>(SELL_SPMMV_ARGS);
+    spmmv_body<VT, K, U, PIPE, Acc, false, 0, LD>(SELL_SPMMV_ARGS);
 }
 
 // Occupancy: the one-vector kernel asks for 4 resident blocks of 512 threads,
@@ -65,14 +65,14 @@ __global__ void __launch_bounds__(512) k_spmmv(SELL_SPMMV_PARAMS) {
 // (unroll 4, pipelined) 319 -> 295 us; bfloat16 unchanged.  The other
 // kernels keep the allocation ptxas picks (capping the wider ones spills
 // hundreds of bytes).
-template <class VT, int U, bool PIPE, class Acc>
+template <class VT, int U, bool PIPE, class Acc, int CT = 0, class LD = Pitch>
 __global__ void __launch_bounds__(512, 4) k_spmv_short(SELL_SPMMV_PARAMS) {
-    spmmv_body<VT, 1, U, PIPE, Acc>(SELL_SPMMV_ARGS);
+    spmmv_body<VT, 1, U, PIPE, Acc, false, CT, LD>(SELL_SPMMV_ARGS);
 }
 
-template <class VT, int K, int U, bool PIPE, int MINB, class Acc>
+template <class VT, int K, int U, bool PIPE, int MINB, class Acc, class LD = Pitch>
 __global__ void __launch_bounds__(512, MINB) k_spmmv_pattern(SELL_SPMMV_PARAMS) {
-    spmmv_body<VT, K, U, PIPE, Acc, true>(SELL_SPMMV_ARGS);
+    spmmv_body<VT, K, U, PIPE, Acc, true, 0, LD>(SELL_SPMMV_ARGS);
 }
 
 #undef SELL_SPMMV_PARAMS
@@ -82,31 +82,25 @@ template <class VT, int K, class AccL>
 cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc, int vec,
                      void *part, int32_t *cnt, int32_t *cnt2, cudaStream_t s) {
     using XT = typename XType<VT>::T;
-    LongArgs a;
-    a.col = h->col;
-    a.cs = h->cs;
-    a.srl = h->srl;
-    a.perm = (h->flags & SELL_BUILD_PERMUTE_COLS) ? nullptr : h->perm;
-    a.lchunk = h->lchunk;
-    a.lrow = h->lrow;
-    a.lunit = h->lunit;
-    a.lwork = h->lwork;
-    a.lmeta = h->lmeta;
-    a.lcol = h->lcol;
-    a.pt = Pattern{h->scol, h->sflag, h->cl};
-    a.nwork = h->lwork ? h->nlwork : h->nunits;
-    a.N = h->nrows;
-    a.C = h->C;
+    const bool wide = ldx >= kWidePitch, pat = h->scol != nullptr && !wide;
+    const LongArgs a = long_args(h, pat);
     const VT *val = static_cast<const VT *>(h->val);
+    const VT *lval = static_cast<const VT *>(h->lval);
     const XT *x = static_cast<const XT *>(X);
     XT *y = static_cast<XT *>(Y);
-    const bool pat = h->scol != nullptr && ldx < (1 << 28);
     constexpr int U = K == 1 ? 8 : (K == 2 ? 4 : 2);
     constexpr bool P = K > 2;
-    const int64_t threads = h->lwork ? h->nlwork * 32 : h->nunits * h->C;
-    auto kern = pat ? k_long<VT, K, U, P, AccL, true> : k_long<VT, K, U, P, AccL, false>;
-    kern<<<(unsigned)((threads + kLongThreads - 1) / kLongThreads), kLongThreads, 0, s>>>(
-        val, static_cast<const VT *>(h->lval), a, part, cnt, cnt2, x, ldx, y, ldy, acc, vec);
+    const unsigned blocks = (unsigned)((long_threads(h) + kLongThreads - 1) / kLongThreads);
+    if constexpr (K == 1) {
+        if (wide) {
+            k_long<VT, 1, 1, false, AccL, false, WidePitch><<<blocks, kLongThreads, 0, s>>>(
+                val, lval, a, part, cnt, cnt2, x, ldx, y, ldy, acc, vec);
+            return cudaGetLastError();
+        }
+    }
+    auto kern = pat ? k_long<VT, K, U, P, AccL, true, Pitch> : k_long<VT, K, U, P, AccL, false, Pitch>;
+    kern<<<blocks, kLongThreads, 0, s>>>(val, lval, a, part, cnt, cnt2, x, Pitch{(int32_t)(ldx * sizeof(XT))}, y, ldy,
+                                         acc, vec);
     return cudaGetLastError();
 }
 
@@ -117,9 +111,9 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
 constexpr int kBlock = 128;
 
 // One launch of a short-row kernel, behind the long rows' where there are any.
-template <class VT, class Kernel>
-cudaError_t launch_short(Kernel kern, const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc,
-                         int vec, cudaStream_t s) {
+template <class VT, class LD, class Kernel>
+cudaError_t launch_short_with(Kernel kern, const sell_matrix *h, const void *X, LD ldx, void *Y, int64_t ldy, int acc,
+                              int vec, cudaStream_t s) {
     using XT = typename XType<VT>::T;
     const VT *val = static_cast<const VT *>(h->val);
     const int32_t *perm = (h->flags & SELL_BUILD_PERMUTE_COLS) ? nullptr : h->perm;
@@ -145,6 +139,12 @@ cudaError_t launch_short(Kernel kern, const sell_matrix *h, const void *X, int64
     return cudaLaunchKernelEx(&cfg, kern, val, static_cast<const int32_t *>(h->col),
                               static_cast<const int64_t *>(h->cs), static_cast<const int32_t *>(h->srl), perm, pt, x,
                               ldx, y, ldy, h->nrows, (int)h->C, acc, vec, 1);
+}
+template <class VT, class Kernel>
+cudaError_t launch_short(Kernel kern, const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc,
+                         int vec, cudaStream_t s) {
+    const Pitch p{(int32_t)(ldx * (int64_t)sizeof(typename XType<VT>::T))};
+    return launch_short_with<VT, Pitch>(kern, h, X, p, Y, ldy, acc, vec, s);
 }
 
 template <class VT, int K, int U, bool PIPE, class Acc>
@@ -215,10 +215,19 @@ cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
         const cudaError_t e = run_long<VT, K, AccL>(h, X, ldx, Y, ldy, acc, vec, part, cnt, cnt2, s);
         if (e != cudaSuccess) return e;
     }
-    if (h->scol && ldx < (1 << 28))  // row pitches beyond 2^31 bytes keep the general kernels
-        return run_pattern<VT, K, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+    if constexpr (K == 1) {
+        if (ldx >= kWidePitch)
+            return launch_short_with<VT, WidePitch>(k_spmv_short<VT, 1, false, Acc, 0, WidePitch>, h, X, ldx, Y, ldy, acc,
+                                                    vec, s);
+    }
+    if (h->scol) return run_pattern<VT, K, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     // (launch mode 2 is the bulk-staged kernel's: its unroll counts slots)
     if ((h->pipeline != 0 && h->unroll == 0) || h->pipeline == 2) {
+        if constexpr (K == 1) {
+            if (h->C == 32)
+                return launch_short<VT>(k_spmv_short<VT, sizeof(VT) == 8 ? 2 : 4, true, Acc, 32>, h, X, ldx, Y, ldy, acc,
+                                        vec, s);
+        }
         constexpr int U = K == 8 ? 2 : 4;
         return run<VT, K, sizeof(VT) == 8 ? U / 2 : U, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     }
