@@ -25,7 +25,9 @@
  *     callbacks.  Default: stream-ordered allocation (cudaMallocFromPoolAsync
  *     / cudaFreeAsync) from one library-owned memory pool per device, which
  *     keeps freed memory for reuse; sell_free returns the pool's unused
- *     memory to the device.
+ *     memory to the device, except for at most 1 GiB (and at most 1/128 of
+ *     the device's memory) that the next build takes again;
+ *     sell_set_allocator returns all of it.
  *   - Concurrency: a handle's products share its long-row scratch, so
  *     products of one handle must not overlap on the GPU (issue them on one
  *     stream, or order the streams), except that SELL_SPMV_HOST_IO products
@@ -126,7 +128,8 @@ typedef void (*sell_free_fn)(void *ptr, void *ctx, void *stream);
 /* ---------------------------------------------------------------- calls */
 
 /* Install process-wide allocation callbacks (both NULL restores the
- * default).  Handles keep the callbacks they were built with. */
+ * default).  Handles keep the callbacks they were built with.  Returns the
+ * unused memory of the library's own pools to their devices. */
 SELL_API sell_status sell_set_allocator(sell_alloc_fn alloc, sell_free_fn release, void *ctx);
 
 /* Convert CRS into SELL-C-sigma (Sec. 3.3 and 3.4, Eqs. "nc", "max"):
