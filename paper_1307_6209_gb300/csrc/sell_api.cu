@@ -295,6 +295,7 @@ sell_status sell_spmv_dot(sell_handle h, const void *x, void *y, uint32_t flags,
     if (flags & (SELL_SPMV_HOST_IO | SELL_SPMV_HOST_DIRECT))
         return fail(SELL_EINVAL, "sell_spmv_dot: device vectors only");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    SELL_TRY(prepare_dot(h, s));
     SELL_TRY(sell_spmmv(h, x, 1, y, 1, 1, flags, stream));
     if (h->nrows == 0) {
         SELL_CUDA_TRY(cudaMemsetAsync(dot, 0, sizeof(double), s));

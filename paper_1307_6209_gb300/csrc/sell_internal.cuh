@@ -141,7 +141,7 @@ struct sell_matrix {
     int32_t bulk_grid = 0, bulk_warps = 0, bulk_ring = 0;
     mutable uint32_t expire_us = 0;  // one-shot test hook of sell_test_expire_wait (0: off),
                                      // consumed by the next bulk-staged launch
-    double *dot_part = nullptr;  // range sums of sell_spmv_dot (lazily allocated)
+    double *dot_part = nullptr;  // range sums and block count of sell_spmv_dot (lazily allocated)
     // host-io staging (lazily allocated): kIoSlots slots used in turn, so that
     // the copies of one call overlap the kernels of the previous ones when
     // calls alternate streams.  A slot is reused only after its result has
@@ -194,6 +194,7 @@ sell_status launch_block_with_scratch(const sell_matrix *h, const void *X, int64
 sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, sell_matrix *h);
 sell_status bulk_plan(sell_matrix *h, int64_t nwarps, cudaStream_t s);
 sell_status bulk_prepare(sell_matrix *h);
+sell_status prepare_dot(sell_matrix *h, cudaStream_t s);
 sell_status launch_dot(sell_matrix *h, const void *x, const void *y, double *out, cudaStream_t s);
 // scratch: per item, batch_item_scratch() bytes of device memory (or NULL for
 // items without long rows); NULL: the plan allocates its own.

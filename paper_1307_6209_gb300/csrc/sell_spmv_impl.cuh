@@ -42,6 +42,7 @@ namespace spmv_impl {
 template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, int CT, class LD>
 __device__ __forceinline__ void spmmv_body(SELL_SPMMV_PARAMS) {
     using XT = typename XType<VT>::T;
+    dependents_may_start();  // a dot product's launch (sell_dot.cu)
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= N) {
         if (after_long) wait_for_predecessor();
