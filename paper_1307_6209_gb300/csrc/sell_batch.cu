@@ -142,12 +142,12 @@ k_batch_rows(const __grid_constant__ RowParams lp) {
 template <class VT, int K, class AccL, class LD = Pitch>
 __global__ void __launch_bounds__(kTileRows) k_batch_long(const __grid_constant__ LongParams lp) {
     using XT = typename XType<VT>::T;
-    constexpr int U = K == 1 ? 8 : (K == 2 ? 4 : 2);
+    constexpr LongShape S = long_shape<VT, K>();
     dependents_may_start();
     const int i = product_of(lp, (int32_t)blockIdx.x);
     if (i < 0) return;
     const LongProd &P = lp.prods[i];
-    long_rows<VT, K, U, (K > 2), AccL, false>(static_cast<const VT *>(P.val), static_cast<const VT *>(P.lval), P.a,
+    long_rows<VT, K, S.unroll, S.pipe, AccL, false>(static_cast<const VT *>(P.val), static_cast<const VT *>(P.lval), P.a,
                                               P.part, P.cnt, P.cnt2, static_cast<const XT *>(P.X), pitch_of<LD>(P),
                                               static_cast<XT *>(P.Y), P.ldy, P.acc, P.vec,
                                               (int64_t)((int32_t)blockIdx.x - lp.start[i]) * blockDim.x + threadIdx.x);

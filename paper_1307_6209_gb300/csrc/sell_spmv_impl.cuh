@@ -79,18 +79,26 @@ __global__ void __launch_bounds__(512, MINB) k_spmmv_pattern(SELL_SPMMV_PARAMS) 
 #undef SELL_SPMMV_PARAMS
 #undef SELL_SPMMV_ARGS
 
+// Where the column patterns are used: several binary64 vectors at once wait
+// for the FP64 pipe, and the pattern kernels' registers cost more than the
+// columns do (100^3 stencil at two vectors 101 us, 94 us without).
+template <class VT, int K>
+constexpr bool pattern_width() {
+    return K == 1 || sizeof(VT) < 8;
+}
+
 template <class VT, int K, class AccL>
 cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc, int vec,
                      void *part, int32_t *cnt, int32_t *cnt2, cudaStream_t s) {
     using XT = typename XType<VT>::T;
-    const bool wide = ldx >= kWidePitch, pat = h->scol != nullptr && !wide;
+    const bool wide = ldx >= kWidePitch, pat = pattern_width<VT, K>() && h->scol != nullptr && !wide;
     const LongArgs a = long_args(h, pat);
     const VT *val = static_cast<const VT *>(h->val);
     const VT *lval = static_cast<const VT *>(h->lval);
     const XT *x = static_cast<const XT *>(X);
     XT *y = static_cast<XT *>(Y);
-    constexpr int U = K == 1 ? 8 : (K == 2 ? 4 : 2);
-    constexpr bool P = K > 2;
+    constexpr int U = long_shape<VT, K>().unroll;
+    constexpr bool P = long_shape<VT, K>().pipe;
     const unsigned blocks = (unsigned)((long_threads(h) + kLongThreads - 1) / kLongThreads);
     if constexpr (K == 1) {
         if (wide) {
@@ -99,7 +107,10 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
             return cudaGetLastError();
         }
     }
-    auto kern = pat ? k_long<VT, K, U, P, AccL, true, Pitch> : k_long<VT, K, U, P, AccL, false, Pitch>;
+    auto kern = k_long<VT, K, U, P, AccL, false, Pitch>;
+    if constexpr (pattern_width<VT, K>()) {
+        if (pat) kern = k_long<VT, K, U, P, AccL, true, Pitch>;
+    }
     kern<<<blocks, kLongThreads, 0, s>>>(val, lval, a, part, cnt, cnt2, x, Pitch{(int32_t)(ldx * sizeof(XT))}, y, ldy,
                                          acc, vec);
     return cudaGetLastError();
@@ -110,6 +121,7 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
 // lengths (2M sorted lognormal rows binary64, unroll 4: block 128 132.7 us,
 // 256 137.4 us, 512 141.7 us; 64 gains nothing more).
 constexpr int kBlock = 128;
+constexpr int64_t kFewRows = 152 * 1024;  // half the chip's threads
 
 // One launch of a short-row kernel, behind the long rows' where there are any.
 template <class VT, class LD, class Kernel>
@@ -172,9 +184,9 @@ cudaError_t run_pattern(const sell_matrix *h, const void *X, int64_t ldx, void *
     constexpr bool F64 = sizeof(VT) == 8;
     auto pick = [&]() {
         if constexpr (K == 1) return k_spmmv_pattern<VT, K, F64 ? 2 : 8, F64, 4, Acc>;
-        else if constexpr (K == 2) return k_spmmv_pattern<VT, K, F64 ? 2 : 4, true, F64 ? 2 : 3, Acc>;
-        else if constexpr (K == 4) return k_spmmv_pattern<VT, K, 4, true, F64 ? 1 : 3, Acc>;
-        else return k_spmmv_pattern<VT, K, F64 ? 2 : 4, true, F64 ? 1 : 2, Acc>;
+        else if constexpr (K == 2) return k_spmmv_pattern<VT, K, 4, true, 3, Acc>;
+        else if constexpr (K == 4) return k_spmmv_pattern<VT, K, 4, true, 3, Acc>;
+        else return k_spmmv_pattern<VT, K, 4, true, 2, Acc>;
     };
     return launch_short<VT>(pick(), h, X, ldx, Y, ldy, acc, vec, s);
 }
@@ -221,7 +233,9 @@ cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
             return launch_short_with<VT, WidePitch>(k_spmv_short<VT, 1, false, Acc, 0, WidePitch>, h, X, ldx, Y, ldy, acc,
                                                     vec, s);
     }
-    if (h->scol) return run_pattern<VT, K, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+    if constexpr (pattern_width<VT, K>()) {
+        if (h->scol) return run_pattern<VT, K, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+    }
     // (launch mode 2 is the bulk-staged kernel's: its unroll counts slots)
     if ((h->pipeline != 0 && h->unroll == 0) || h->pipeline == 2) {
         if constexpr (K == 1) {
@@ -230,6 +244,13 @@ cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
                                         vec, s);
         }
         constexpr int U = K == 8 ? 2 : 4;
+        if constexpr (K == 2 && sizeof(VT) == 8) {
+            // few or even rows like the loads in flight better than the warps:
+            // 20,000 banded rows 6.8 us with unroll 4, 9.6 us with 2, 250,000
+            // 30.1 and 32.3 us, 100^3 stencil 94 and 96 us; 1M lognormal rows
+            // 74 and 70 us
+            if (h->nrows <= kFewRows || !h->nunits) return run<VT, K, 4, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+        }
         return run<VT, K, sizeof(VT) == 8 ? U / 2 : U, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     }
     if (h->pipeline != 0) return pick_u<VT, K, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
