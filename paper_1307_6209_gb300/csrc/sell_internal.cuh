@@ -86,6 +86,23 @@ inline int rhs_block(int rem, int maxw) {
 // column at a time, in kernels of their own (sell_rowdot.cuh, WidePitch).
 constexpr int64_t kWidePitch = 1 << 28;
 
+// A block of 3 or of 5 to 7 right-hand sides of binary32 vectors (7 of
+// binary64) runs as one of 4 or 8 on a copy of X with rows of that many
+// values: one vector load per gathered row and one pass over the matrix, where
+// the blocks 2 + 1 or 4 + 2 + 1 take a load per value and a pass each.  The
+// kernels write the first `cols` columns, bits 4-7 of their vec argument (0:
+// all).  Worth a pass over X where a column has at least two entries on
+// average.  Measured at k = 3 / 5 / 7, binary32: 1M lognormal rows 192 / 244 /
+// 357 -> 105 / 129 / 139 us, 500,000 banded rows 50 / 80 / 116 -> 39 / 54 / 58
+// us, 100^3 stencil 92 / 127 / 182 -> 64 / 81 / 85 us.  Binary64 pays for the
+// columns that are not there with the FP64 pipe's time (100^3 stencil at k = 3
+// 160 -> 213 us, at 5 273 -> 380 us) except at 7: 393 -> 381 us, lognormal
+// 505 -> 352 us.
+inline int pad_block(int rem, int maxw, bool f64) {
+    if (rem == 3 && maxw >= 4 && !f64) return 4;
+    return rem >= (f64 ? 7 : 5) && rem <= 7 && maxw >= 8 ? 8 : 0;
+}
+
 // How the kernels may load a row of X, or store a row of Y (base, row pitch
 // ld elements of xs bytes): 2 with 32-byte vectors, 1 with 16-byte vectors,
 // 0 value by value.  The kernels take X's in bits 0-1 and Y's in bits 2-3.
@@ -133,6 +150,7 @@ struct sell_matrix {
     int32_t *cnt2 = nullptr;   // nunits * C group counters of very long rows (zero at rest)
     void *part = nullptr;      // segment partials: nunits * C * part_k * 8 bytes
     int32_t part_k = 0;
+    void *xpad = nullptr;      // padded copy of X (pad_block): ncols * 8 values, allocated on first use
     // bulk-staged SpMV (launch mode 2), prepared by sell_set_launch
     int32_t *bsc = nullptr;    // nchunks staged columns per chunk
     int32_t *wsplit = nullptr; // wsplit_n + 1 per-warp chunk boundaries
@@ -184,6 +202,13 @@ struct sell_batch {
 
 namespace sell {
 
+// Three columns trade one launch for another, which a small matrix of short
+// rows is not worth (20^3 stencil 14.4 -> 16.2 us; 5000 lognormal rows, with
+// long ones, 41 -> 21 us).
+inline bool pad_pays(const sell_matrix *h, int cols) {
+    return h->ncols > 0 && h->nnz >= 2 * h->ncols && (cols > 3 || h->nunits > 0 || h->nnz >= 500000);
+}
+
 // --------------------------------------------------------- launch entry points
 // (defined in sell_spmv.cu / sell_build.cu / sell_batch.cu / sell_bench.cu)
 sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy,
@@ -191,6 +216,8 @@ sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, in
 sell_status launch_block_with_scratch(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
                                       int64_t ldy, int kb, uint32_t flags, void *part, int32_t *cnt,
                                       int32_t *cnt2, cudaStream_t s);
+// dst (n x K, dense) = the first cols values of every row of X (n rows, ldx apart), zeros behind them.
+cudaError_t launch_pad(const void *X, int64_t ldx, int64_t n, int cols, int K, size_t xs, void *dst, cudaStream_t s);
 sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, sell_matrix *h);
 sell_status bulk_plan(sell_matrix *h, int64_t nwarps, cudaStream_t s);
 sell_status bulk_prepare(sell_matrix *h);

@@ -198,7 +198,7 @@ __device__ __forceinline__ void fold_warp(bool done, const PT *part, int64_t bas
 // complete.  All 32 lanes call; acc counts where g.valid.
 template <class XT, int K, class Acc>
 __device__ __forceinline__ void long_finish(const LongArgs &a, const LongSeg &g, const Acc (&acc)[K], void *part,
-                                            int32_t *cnt, int32_t *cnt2, XT *Y, int64_t ldy) {
+                                            int32_t *cnt, int32_t *cnt2, XT *Y, int64_t ldy, int vec) {
     using PT = typename PartOf<Acc>::T;
     PT *pp = static_cast<PT *>(part);
     const int C = a.C;
@@ -240,7 +240,8 @@ __device__ __forceinline__ void long_finish(const LongArgs &a, const LongSeg &g,
     if (done) {
         const int64_t out = a.perm ? (int64_t)a.perm[g.r] : g.r;
 #pragma unroll
-        for (int q = 0; q < K; ++q) Y[out * ldy + q] = static_cast<XT>(tot[q].result());
+        for (int q = 0; q < K; ++q)
+            if (has_column<K>(q, vec)) Y[out * ldy + q] = static_cast<XT>(tot[q].result());
         *ct = 0;
     }
 }
@@ -280,7 +281,8 @@ __device__ __forceinline__ void long_rows(const VT *__restrict__ val, const VT *
     if (g.valid) {
         const int64_t out = a.perm ? (int64_t)a.perm[g.r] : g.r;
 #pragma unroll
-        for (int q = 0; q < K; ++q) acc[q].init((g.s == 0 && accumulate) ? Y[out * ldy + q] : XT(0));
+        for (int q = 0; q < K; ++q)
+            acc[q].init((g.s == 0 && accumulate && has_column<K>(q, vec)) ? Y[out * ldy + q] : XT(0));
         const int n = min(g.L - g.s * kSeg, kSeg);
         const VT *vp = (g.packed ? lval : val) + g.base;
         bool done = false;
@@ -289,16 +291,16 @@ __device__ __forceinline__ void long_rows(const VT *__restrict__ val, const VT *
                 const int64_t cs0 = a.cs[g.c];
                 const int32_t *op = a.pt.off + offset_start(cs0, a.pt.cl[g.c], g.l >> 5, g.r >> 5) + g.s * kSeg;
                 chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, vp, op, __ldg(a.col + cs0 + g.l), g.stride, 0, n, X,
-                                                          ldx, vec & 3, pol);
+                                                          ldx, vec, pol);
                 done = true;
             }
         }
         if (!done)
             chain<VT, XT, K, U, PIPE, Acc>(acc, vp, (g.packed ? a.lcol : a.col) + g.base, g.stride, 0, n, X, ldx,
-                                           vec & 3, pol);
+                                           vec, pol);
     }
     __syncwarp();
-    long_finish<XT, K, Acc>(a, g, acc, part, cnt, cnt2, Y, ldy);
+    long_finish<XT, K, Acc>(a, g, acc, part, cnt, cnt2, Y, ldy, vec);
 }
 
 template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, class LD>

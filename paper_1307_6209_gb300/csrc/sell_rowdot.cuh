@@ -213,6 +213,21 @@ __device__ __forceinline__ void ld_y32(const double *p, double *v) {
                  : "memory");
 }
 
+// The columns of a block of K that are there (bits 4-7 of vec, 0: all; fewer
+// only with bits 2-3 zero), and whether column q is: the smallest numbers that
+// pad_block puts in a block are known.
+template <int K>
+__device__ __forceinline__ int columns(int vec) {
+    if constexpr (K < 4) return K;
+    const int n = (vec >> 4) & 15;
+    return n ? n : K;
+}
+template <int K>
+__device__ __forceinline__ bool has_column(int q, int vec) {
+    if constexpr (K < 4) return true;
+    return q < (K == 4 ? 3 : 5) || q < columns<K>(vec);
+}
+
 // Row i of Y (K values, row-major, ldy) written, or read for accumulation,
 // with the widest vectors that bits 2-3 of vec allow (the layout of load_x).
 // One vector store per 32 bytes instead of K scalar stores: each scalar
@@ -239,8 +254,10 @@ __device__ __forceinline__ void store_y(XT *Y, int64_t ldy, int64_t i, int vec, 
                     *reinterpret_cast<float4 *>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
             }
         } else {
+            const int n = columns<K>(vec);
 #pragma unroll
-            for (int q = 0; q < K; ++q) p[q] = v[q];
+            for (int q = 0; q < K; ++q)
+                if (q < n) p[q] = v[q];
         }
     }
 }
@@ -275,8 +292,9 @@ __device__ __forceinline__ void load_y(const XT *Y, int64_t ldy, int64_t i, int 
                 }
             }
         } else {
+            const int n = columns<K>(vec);
 #pragma unroll
-            for (int q = 0; q < K; ++q) v[q] = p[q];
+            for (int q = 0; q < K; ++q) v[q] = q < n ? p[q] : XT(0);
         }
     }
 }
@@ -651,7 +669,7 @@ __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int3
 #pragma unroll
         for (int q = 0; q < K; ++q) acc[q].init(XT(0));
     }
-    row_chain<VT, XT, K, U, PIPE, Acc, PAT, CT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec & 3, pol);
+    row_chain<VT, XT, K, U, PIPE, Acc, PAT, CT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec, pol);
     XT yo[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) yo[q] = acc[q].result();

@@ -3,6 +3,8 @@
 // and dispatches to the per-type kernels (sell_spmv_impl.cuh, instantiated in
 // sell_spmv_f64.cu, sell_spmv_f32.cu, sell_spmv_bf16.cu).
 
+#include <algorithm>
+
 #include "sell_internal.cuh"
 
 namespace sell {
@@ -30,36 +32,90 @@ cudaError_t dispatch(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
     }
 }
 
+// One thread per value of the padded rows: reads and writes run along the rows.
+template <class T>
+__global__ void __launch_bounds__(256) k_pad(const T *__restrict__ X, int64_t ldx, int64_t n, int cols, int K,
+                                             T *__restrict__ dst) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * K; i += stride) {
+        const int64_t row = K == 4 ? i >> 2 : i >> 3;
+        const int q = (int)(i & (K - 1));
+        dst[i] = q < cols ? X[row * ldx + q] : T(0);
+    }
+}
+
+bool grow_part(sell_matrix *h, int need, cudaStream_t s) {
+    void *p = h->al.get((size_t)h->nunits * h->C * need * 8, s);
+    if (!p) return false;
+    h->al.put(h->part, s);
+    h->part = p;
+    h->part_k = need;
+    return true;
+}
+
+// Memory for padded blocks of `width` columns: the copy of X, once per handle
+// and for the widest block, so that a captured graph's pointer stays good;
+// the long rows' scratch.  Allocates nothing while the stream is captured (the
+// blocks 4, 2, 1 need neither).
+bool make_pad(sell_matrix *h, int width, cudaStream_t s) {
+    const bool part = h->nunits > 0 && width > h->part_k;
+    if (!h->xpad || part) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        if (st != cudaStreamCaptureStatusNone) return false;
+    }
+    if (!h->xpad) h->xpad = h->al.get((size_t)h->ncols * 8 * (h->store_type == SELL_F64 ? 8 : 4), s);
+    return h->xpad && (!part || grow_part(h, width, s));
+}
+
 }  // namespace
 
+cudaError_t launch_pad(const void *X, int64_t ldx, int64_t n, int cols, int K, size_t xs, void *dst, cudaStream_t s) {
+    const unsigned grid = (unsigned)std::min<int64_t>((n * K + 255) / 256, 152 * 64);
+    if (xs == 8)
+        k_pad<double><<<grid, 256, 0, s>>>(static_cast<const double *>(X), ldx, n, cols, K, static_cast<double *>(dst));
+    else
+        k_pad<float><<<grid, 256, 0, s>>>(static_cast<const float *>(X), ldx, n, cols, K, static_cast<float *>(dst));
+    return cudaGetLastError();
+}
+
 // Splits k into kernel blocks of 8, 4, 2, 1 columns, at most the flags' block
-// width (every column keeps the same per-row operation order, so the split
-// does not change any result).  The segment scratch grows on the first
+// width, and odd numbers of last columns into one padded block (every column
+// keeps the same per-row operation order, so the split does not change any
+// result).  The segment scratch grows on the first
 // product with a wider block.
 sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy,
                          int32_t k, uint32_t flags, cudaStream_t s) {
     if (h->nrows == 0) return SELL_OK;
     const int maxw = ldx < kWidePitch ? max_rhs_block(flags) : 1;
-    if (h->nunits > 0) {
-        const int need = rhs_block(k, maxw);
-        if (need > h->part_k) {
-            void *p = h->al.get((size_t)h->nunits * h->C * need * 8, s);
-            if (!p) return fail(SELL_ENOMEM, "segment scratch allocation failed");
-            h->al.put(h->part, s);
-            h->part = p;
-            h->part_k = need;
-        }
-    }
+    const size_t xs = h->store_type == SELL_F64 ? 8 : 4;
+    const int last = k % 8, odd = pad_block(last, maxw, h->store_type == SELL_F64), plain = rhs_block(k, maxw);
+    const bool pad = odd && pad_pays(h, last) && make_pad(h, std::max(odd, plain), s);
+    const int need = pad ? std::max(odd, plain) : plain;
+    if (h->nunits > 0 && need > h->part_k && !grow_part(h, need, s))
+        return fail(SELL_ENOMEM, "segment scratch allocation failed");
     const int acc = (flags & SELL_SPMV_ACCUMULATE) ? 1 : 0;
     const int comp = comp_mode(flags);
-    const size_t xs = h->store_type == SELL_F64 ? 8 : 4;
     int32_t done = 0;
     while (done < k) {
-        const int kb = rhs_block(k - done, maxw);
+        const int rem = k - done;
         const char *Xb = static_cast<const char *>(X) + (size_t)done * xs;
         char *Yb = static_cast<char *>(Y) + (size_t)done * xs;
+        cudaError_t e;
+        if (pad && rem == last) {
+            e = launch_pad(Xb, ldx, h->ncols, rem, odd, xs, h->xpad, s);
+            if (e == cudaSuccess)
+                e = dispatch(h, h->xpad, odd, Yb, ldy, odd, acc, x_vec(h->xpad, odd, xs) | (rem << 4), comp, nullptr,
+                             nullptr, nullptr, s);
+            if (e != cudaSuccess) return cuda_fail(e, "SpMV kernel launch");
+            break;
+        }
+        const int kb = rhs_block(rem, maxw);
         int vec = x_vec(Xb, ldx, xs) | (x_vec(Yb, ldy, xs) << 2);
-        cudaError_t e = dispatch(h, Xb, ldx, Yb, ldy, kb, acc, vec, comp, nullptr, nullptr, nullptr, s);
+        e = dispatch(h, Xb, ldx, Yb, ldy, kb, acc, vec, comp, nullptr, nullptr, nullptr, s);
         if (e != cudaSuccess) return cuda_fail(e, "SpMV kernel launch");
         done += kb;
     }
