@@ -28,7 +28,8 @@
  *     memory to the device, except for at most 1 GiB (and at most 1/128 of
  *     the device's memory) that the next build takes again;
  *     sell_set_allocator returns all of it.
- *   - Concurrency: a handle's products share its long-row scratch, so
+ *   - Concurrency: a handle's products share its long-row scratch (and a
+ *     padded copy of X at 3 and 5 to 7 right-hand sides), so
  *     products of one handle must not overlap on the GPU (issue them on one
  *     stream, or order the streams), except that SELL_SPMV_HOST_IO products
  *     are ordered by the library, and sell_spmmv_noalloc / batch plans use
@@ -221,7 +222,10 @@ SELL_API sell_status sell_spmv_dot(sell_handle h, const void *x, void *y, uint32
  * once for up to 8 vectors).  X is ncols x k and Y nrows x k, row-major with
  * leading dimensions ldx >= k and ldy >= k (in elements); element types as in
  * sell_spmv.  k > 8 is processed in blocks of 8 columns, streaming the
- * matrix once per block.  Column c of Y equals sell_spmv of column c of X
+ * matrix once per block; 3 and 5 to 7 columns of binary32 vectors (7 of
+ * binary64) are one block too, on a copy of X with padded rows that the handle
+ * allocates on their first use (without the memory, or while the stream is
+ * captured, blocks of 4, 2 and 1 are used).  Column c of Y equals sell_spmv of column c of X
  * bit for bit.  Errors as sell_spmv, plus SELL_EINVAL for k < 1, ldx < k,
  * ldy < k. */
 SELL_API sell_status sell_spmmv(sell_handle h, const void *X, int64_t ldx, void *Y, int64_t ldy,
@@ -232,8 +236,9 @@ SELL_API sell_status sell_spmmv(sell_handle h, const void *X, int64_t ldx, void 
  * memory at the time they multiply -- a serving loop held to a fixed memory
  * budget, code running inside another framework's memory pool, or a
  * latency-critical path that must not wait for an allocation.  (sell_spmmv
- * itself may allocate: staging buffers for SELL_SPMV_HOST_IO, and a larger
- * long-row scratch the first time a call uses more right-hand sides.)
+ * itself may allocate: staging buffers for SELL_SPMV_HOST_IO, a larger
+ * long-row scratch the first time a call uses more right-hand sides, and a
+ * padded copy of X the first time it uses 3 or 5 to 7.)
  * Instead of memory owned by the handle, the partial sums of long rows
  * (rows longer than 64 entries) go to one fixed 4 MiB device array that the
  * library holds on every device where it is loaded, until the process exits.

@@ -1,5 +1,6 @@
-// sell_long.cuh -- the rows longer than kSeg of a single product, in a kernel
-// of their own that runs ahead of the short rows' (sell_spmv_impl.cuh).
+// sell_long.cuh -- the rows longer than kSeg of single products and batches, in
+// kernels of their own that run ahead of the short rows' (sell_spmv_impl.cuh,
+// sell_batch.cu).
 //
 // Work: lwork lists the virtual warps (LongWork).  In a chunk of mostly long
 // rows (mode 0) a virtual warp takes one segment of 32 neighbouring rows; in
