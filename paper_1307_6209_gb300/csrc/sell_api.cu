@@ -135,7 +135,7 @@ void free_matrix(sell_matrix *h) {
     (void)cudaDeviceSynchronize();
     void *ptrs[] = {h->val,    h->col,   h->cs,   h->cl,     h->srl,    h->perm,
                     h->lchunk, h->lunit, h->cnt, h->cnt2, h->part, h->bsc, h->wsplit, h->dstat, h->dot_part,
-                    h->lrow,   h->lmeta, h->scol, h->sflag, h->lwork, h->lval, h->lcol, h->xpad};
+                    h->lrow,   h->lmeta, h->scol, h->sflag, h->lwork, h->lval, h->lcol, h->xpad, h->ppad};
     for (void *p : ptrs) h->al.put(p, nullptr);
     for (auto &sl : h->io) {
         h->al.put(sl.x, nullptr);

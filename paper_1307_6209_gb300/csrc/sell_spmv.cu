@@ -4,6 +4,7 @@
 // sell_spmv_f64.cu, sell_spmv_f32.cu, sell_spmv_bf16.cu).
 
 #include <algorithm>
+#include <mutex>
 
 #include "sell_internal.cuh"
 
@@ -53,22 +54,23 @@ bool grow_part(sell_matrix *h, int need, cudaStream_t s) {
     return true;
 }
 
-// Memory for padded blocks of `width` columns: the copy of X, once per handle
-// and for the widest block, so that a captured graph's pointer stays good;
-// the long rows' scratch.  Allocates nothing while the stream is captured (the
-// blocks 4, 2, 1 need neither).
-bool make_pad(sell_matrix *h, int width, cudaStream_t s) {
-    const bool part = h->nunits > 0 && width > h->part_k;
-    if (!h->xpad || part) {
-        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return false;
-        }
-        if (st != cudaStreamCaptureStatusNone) return false;
+// Memory for padded blocks: the copy of X and a long-row scratch of their own,
+// once per handle and for the widest block.  Neither ever moves, and h->part
+// does not grow for a padded block, so the pointers in a captured graph stay
+// good whatever widths run after it.  Allocates nothing while the stream is
+// captured (the blocks 4, 2, 1 need neither).
+bool make_pad(sell_matrix *h, cudaStream_t s) {
+    const bool part = h->nunits > 0 && !h->ppad;
+    if (h->xpad && !part) return true;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
     }
+    if (st != cudaStreamCaptureStatusNone) return false;
+    if (part && !(h->ppad = h->al.get((size_t)h->nunits * h->C * 8 * 8, s))) return false;
     if (!h->xpad) h->xpad = h->al.get((size_t)h->ncols * 8 * (h->store_type == SELL_F64 ? 8 : 4), s);
-    return h->xpad && (!part || grow_part(h, width, s));
+    return h->xpad != nullptr;
 }
 
 }  // namespace
@@ -93,8 +95,12 @@ sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, in
     const int maxw = ldx < kWidePitch ? max_rhs_block(flags) : 1;
     const size_t xs = h->store_type == SELL_F64 ? 8 : 4;
     const int last = k % 8, odd = pad_block(last, maxw, h->store_type == SELL_F64), plain = rhs_block(k, maxw);
-    const bool pad = odd && pad_pays(h, last) && make_pad(h, std::max(odd, plain), s);
-    const int need = pad ? std::max(odd, plain) : plain;
+    // Host threads may issue products of one handle on one stream: another
+    // thread's copy must not come between this one's copy and its product.
+    std::unique_lock<std::mutex> lock(h->pad_mu, std::defer_lock);
+    if (odd && pad_pays(h, last)) lock.lock();
+    const bool pad = lock.owns_lock() && make_pad(h, s);
+    const int need = pad && k < 8 ? 0 : plain;
     if (h->nunits > 0 && need > h->part_k && !grow_part(h, need, s))
         return fail(SELL_ENOMEM, "segment scratch allocation failed");
     const int acc = (flags & SELL_SPMV_ACCUMULATE) ? 1 : 0;
@@ -108,8 +114,8 @@ sell_status launch_spmmv(sell_matrix *h, const void *X, int64_t ldx, void *Y, in
         if (pad && rem == last) {
             e = launch_pad(Xb, ldx, h->ncols, rem, odd, xs, h->xpad, s);
             if (e == cudaSuccess)
-                e = dispatch(h, h->xpad, odd, Yb, ldy, odd, acc, x_vec(h->xpad, odd, xs) | (rem << 4), comp, nullptr,
-                             nullptr, nullptr, s);
+                e = dispatch(h, h->xpad, odd, Yb, ldy, odd, acc, x_vec(h->xpad, odd, xs) | (rem << 4), comp, h->ppad,
+                             h->cnt, h->cnt2, s);
             if (e != cudaSuccess) return cuda_fail(e, "SpMV kernel launch");
             break;
         }

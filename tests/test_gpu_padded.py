@@ -104,3 +104,62 @@ def test_failing_allocation_takes_the_narrow_blocks():
         assert torch.equal(*got)
     finally:
         assert lib.sell_set_allocator(sell.ALLOC_FN(), sell.FREE_FN(), None) == sell.SELL_OK
+
+
+@pytest.mark.parametrize("store", [0, 1])
+def test_padded_widths_leave_a_captured_graphs_scratch(store):
+    """A graph of two columns, captured with the long rows' scratch at two:
+    padded widths after it neither move nor free that scratch."""
+    import torch
+    from paper_1307_6209_gb300 import sell
+    A = MATS[0][1]
+    dt = torch.float64 if store == 0 else torch.float32
+    X = torch.from_numpy(synth.block(A.ncols, 7, seed=8)).to(dt).cuda()
+    h = sell.sell_build(A, C=32, store_type=store)
+    x2, y2 = X[:, :2].contiguous(), torch.zeros((A.nrows, 2), dtype=dt, device="cuda")
+    sell.sell_spmmv(h, x2, y2)
+    want = y2.clone()
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        sell.sell_spmmv(h, x2, y2)
+    y7 = torch.zeros((A.nrows, 7), dtype=dt, device="cuda")
+    sell.sell_spmmv(h, X, y7)
+    if store:
+        sell.sell_spmmv(h, X[:, :3].contiguous(), torch.zeros((A.nrows, 3), dtype=dt, device="cuda"))
+    torch.cuda.synchronize()
+    for _ in range(3):
+        y2.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y2, want) and torch.equal(y7[:, :2], want)
+    h.free()
+
+
+def test_threads_on_one_stream_keep_their_padded_copies():
+    import threading
+    import torch
+    from paper_1307_6209_gb300 import sell
+    A = MATS[1][1]
+    h = sell.sell_build(A, C=32, store_type=1)
+    Xs = [torch.from_numpy(synth.block(A.ncols, 5, seed=20 + t)).float().cuda() for t in range(4)]
+    ref = sell.sell_build(A, C=32, store_type=1)
+    want = []
+    for X in Xs:
+        y = torch.empty((A.nrows, 5), device="cuda")
+        sell.sell_spmmv(ref, X, y)
+        want.append(y)
+    ys = [[torch.zeros((A.nrows, 5), device="cuda") for _ in range(200)] for _ in Xs]
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def work(t):
+        with torch.cuda.stream(stream):
+            for y in ys[t]:
+                sell.sell_spmmv(h, Xs[t], y)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    torch.cuda.synchronize()
+    assert all(torch.equal(y, w) for l, w in zip(ys, want) for y in l)
