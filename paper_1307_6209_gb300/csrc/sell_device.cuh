@@ -46,9 +46,19 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
     return p;
 }
 
-// Ask L2 for `bytes` (a multiple of 16) at p (16-byte aligned), one request.
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes, uint64_t pol) {
-    asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p), "r"(bytes), "l"(pol));
+// Where `ask` holds, ask L2 for `bytes` (a multiple of 16) at p (16-byte
+// aligned), one request.  A predicated instruction and not a branch: behind a
+// branch that one lane takes, the warp can stay split, and what follows is
+// issued twice (the column-pattern kernels, which ask with one lane: with the
+// slice's flag loaded ahead of the branch 271 us on the 150^3 stencil binary32
+// at eight vectors, behind it 183, predicated 166; 187^3 bfloat16 181, 153, 145).
+__device__ __forceinline__ void prefetch_l2(bool ask, const void *p, uint32_t bytes, uint64_t pol) {
+    asm volatile(
+        "{\n"
+        ".reg .pred ask;\n"
+        "setp.ne.s32 ask, %3, 0;\n"
+        "@ask cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;\n"
+        "}" ::"l"(p), "r"(bytes), "l"(pol), "r"((int)ask));
 }
 
 __device__ __forceinline__ double ld_stream(const double *ptr, uint64_t pol) {

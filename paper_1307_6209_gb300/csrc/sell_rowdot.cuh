@@ -516,8 +516,9 @@ __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ 
         const int n = j1 - j0;
         const int64_t at = cs0 + (int64_t)j0 * C + (int64_t)(l & ~31) * n;
         const bool ask = PREFETCH && (l & 31) == 0 && n > 0;
-        if (ask) prefetch_l2(val + at, (uint32_t)(n * 32 * sizeof(VT)), pol);
-        if (pt.flag[r >> 5]) {
+        const int32_t flag = pt.flag[r >> 5];
+        prefetch_l2(ask, val + at, (uint32_t)(n * 32 * sizeof(VT)), pol);
+        if (flag) {
             if (n <= 0) return;
             const int32_t first = __ldg(col + base);
             const int32_t *op = pt.off + offset_start(cs0, width, l >> 5, r >> 5);
@@ -530,7 +531,7 @@ __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ 
             chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
             return;
         }
-        if (ask) prefetch_l2(col + at, (uint32_t)(n * 128), pol);
+        prefetch_l2(ask, col + at, (uint32_t)(n * 128), pol);
     }
     chain<VT, XT, K, U, PIPE, Acc, CT>(acc, val + base, col + base, C, j0, j1, X, ldx, vec, pol);
 }

@@ -171,21 +171,22 @@ cudaError_t run(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64
 // and one offset per 32 entries instead of 32 columns, and the gathers no
 // longer wait for streamed columns.  Bound: HBM for the values (binary64 at
 // one vector: the FP64 pipe, 348 us on the 200^3 stencil).  Measured, block
-// 128, before -> after: 200^3 stencil binary64 423 -> 375 us; 187^3 binary32
-// 219 -> 170 us and bfloat16 212 -> 152 us (best launch before); 150^3
-// binary32 at k = 4 / 8 206 (k = 8) -> 136 / 184 us; dense 3000^2 binary32
+// 128, before -> after: 200^3 stencil binary64 423 -> 374 us; 187^3 binary32
+// 219 -> 167 us and bfloat16 212 -> 145 us (best launch before); 150^3
+// binary32 at k = 4 / 8 206 (k = 8) -> 137 / 166 us; dense 3000^2 binary32
 // 18.8 -> 16.6 us.  Unroll, pipelining and resident blocks per width were
 // swept on these; more loads in flight per thread cost registers, and the
 // kernel loses more warps than it gains loads (binary64 with unroll 8:
-// 437 us; k = 8 with 3 blocks: 438 us, spills).
+// 437 us; k = 8 with 3 blocks: 438 us, spills; k = 8 with unroll 2 168 us, not
+// pipelined 191 us; one binary32 vector with unroll 8 168 us, bfloat16 148 us).
 template <class VT, int K, class Acc>
 cudaError_t run_pattern(const sell_matrix *h, const void *X, int64_t ldx, void *Y, int64_t ldy, int acc, int vec,
                         cudaStream_t s) {
     constexpr bool F64 = sizeof(VT) == 8;
     auto pick = [&]() {
-        if constexpr (K == 1) return k_spmmv_pattern<VT, K, F64 ? 2 : 8, F64, 4, Acc>;
+        if constexpr (K == 1) return k_spmmv_pattern<VT, K, F64 ? 2 : 4, F64, 4, Acc>;
         else if constexpr (K == 2) return k_spmmv_pattern<VT, K, 4, true, 3, Acc>;
-        else if constexpr (K == 4) return k_spmmv_pattern<VT, K, 4, true, 3, Acc>;
+        else if constexpr (K == 4) return k_spmmv_pattern<VT, K, 4, false, 3, Acc>;
         else return k_spmmv_pattern<VT, K, 4, true, 2, Acc>;
     };
     return launch_short<VT>(pick(), h, X, ldx, Y, ldy, acc, vec, s);
