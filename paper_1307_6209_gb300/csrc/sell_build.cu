@@ -398,6 +398,12 @@ sell_status scan_exclusive(const T *in, int64_t n, int64_t *out, const Allocator
 // The sums over the chunks in one scan: chunk offsets (C * cl), long chunks
 // (cl > kSeg), their segments (ceil(cl / kSeg) each), the virtual warps of
 // sell_long.cuh and those of them with packed entries.  nlr[c] = rows of chunk c longer than kSeg.
+// The first long-row warp and pack of a chunk (8-byte aligned, as an allocator's
+// memory may be).
+struct WorkBase {
+    int64_t nwork, npack;
+};
+
 struct ChunkSums {
     int64_t stored, nlong, nunits, nwork, npack;
     __device__ __forceinline__ ChunkSums &operator+=(const ChunkSums &o) {
@@ -470,7 +476,7 @@ __global__ void __launch_bounds__(kScanThreads)
 k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, int64_t Nc, int64_t per, int C,
               const ChunkSums *__restrict__ tile,
               int64_t *__restrict__ cs, int64_t *__restrict__ lpos, int64_t *__restrict__ ubase,
-              longlong2 *__restrict__ wbase, ChunkSums *__restrict__ total) {
+              WorkBase *__restrict__ wbase, ChunkSums *__restrict__ total) {
     __shared__ ChunkSums wt[32];
     __shared__ ChunkSums before;
     ChunkSums s = {0, 0, 0, 0, 0};
@@ -488,7 +494,7 @@ k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, i
             cs[c] = v.stored - own.stored;
             lpos[c] = v.nlong - own.nlong;
             ubase[c] = v.nunits - own.nunits;
-            wbase[c] = make_longlong2(v.nwork - own.nwork, v.npack - own.npack);
+            wbase[c] = WorkBase{v.nwork - own.nwork, v.npack - own.npack};
             if (c == Nc - 1) {
                 cs[Nc] = v.stored;
                 *total = v;
@@ -553,7 +559,7 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
 // lane of the row), so the results do not depend on the mode.
 __global__ void __launch_bounds__(256)
 k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, const int64_t *__restrict__ lpos,
-             const int64_t *__restrict__ ubase, const longlong2 *__restrict__ wbase, const int64_t *__restrict__ cs, int64_t Nc, int64_t N, int C,
+             const int64_t *__restrict__ ubase, const WorkBase *__restrict__ wbase, const int64_t *__restrict__ cs, int64_t Nc, int64_t N, int C,
              int32_t *__restrict__ lchunk, int2 *__restrict__ lunit, int32_t *__restrict__ lrow,
              int4 *__restrict__ lmeta, LongWork *__restrict__ lwork) {
     const int lane = threadIdx.x & 31;
@@ -574,7 +580,7 @@ k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, co
     const bool few = few_long(m, C);
     if (lwork) {
         const int64_t n = few ? ((int64_t)m * nseg + 31) / 32 : (int64_t)nseg * (C / 32);
-        const longlong2 wb = wbase[c];
+        const WorkBase wb = wbase[c];
         for (int64_t k = lane; k < n; k += 32) {
             LongWork wk;
             wk.lc = (int32_t)i;
@@ -582,10 +588,10 @@ k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, co
             wk.nseg = nseg;
             wk.m = few ? m : -1;
             const int sl = (int)(k % (C / 32)), sg = (int)(k / (C / 32));
-            wk.base = few ? (wb.y + k) * (kSeg * 32) : cs[c] + (int64_t)sg * kSeg * C + sl * 32;
+            wk.base = few ? (wb.npack + k) * (kSeg * 32) : cs[c] + (int64_t)sg * kSeg * C + sl * 32;
             wk.i = (int32_t)k;
             wk.u0 = (int32_t)u;
-            lwork[wb.x + k] = wk;
+            lwork[wb.nwork + k] = wk;
         }
     }
     if (lane == 0) {
@@ -1115,14 +1121,14 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_TRY(tile.alloc(al, (nt + 1) * sizeof(ChunkSums), s));
         SELL_TRY(lpos.alloc(al, Nc * sizeof(int64_t), s));
         SELL_TRY(ubase.alloc(al, Nc * sizeof(int64_t), s));
-        SELL_TRY(wbase.alloc(al, Nc * sizeof(longlong2), s));
+        SELL_TRY(wbase.alloc(al, Nc * sizeof(WorkBase), s));
         const int32_t *nlr = cl.as<int32_t>() + Nc;
         ChunkSums *tp = tile.as<ChunkSums>();
         k_chunk_reduce<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), nlr, Nc, per, C, tp);
         SELL_CUDA_TRY(cudaGetLastError());
         k_chunk_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), nlr, Nc, per, C, tp, cs.as<int64_t>(),
                                                             lpos.as<int64_t>(), ubase.as<int64_t>(),
-                                                            wbase.as<longlong2>(), tp + nt);
+                                                            wbase.as<WorkBase>(), tp + nt);
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_CUDA_TRY(cudaMemcpyAsync(&total, tp + nt, sizeof(total), cudaMemcpyDeviceToHost, s));
         SELL_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1143,7 +1149,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         }
         k_long_lists<<<(unsigned)((Nc + 7) / 8), 256, 0, s>>>(cl.as<int32_t>(), srl.as<int32_t>(),
                                                                   lpos.as<int64_t>(), ubase.as<int64_t>(),
-                                                                  wbase.as<longlong2>(), cs.as<int64_t>(), Nc, N, C,
+                                                                  wbase.as<WorkBase>(), cs.as<int64_t>(), Nc, N, C,
                                                                   lchunk.as<int32_t>(), lunit.as<int2>(),
                                                                   lrow.as<int32_t>(), lmeta.as<int4>(),
                                                                   lwork.as<LongWork>());
@@ -1205,9 +1211,9 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         // entry have a trivial one; a slice without one reads its columns.)
         unsigned long long nopat = 0;
         for (unsigned long long n : end.nopat) nopat += n;
-        // The kernel loads offsets and prefetches values in 16-byte units.
+        // The kernel loads offsets and prefetches values and columns in 16-byte units.
         pattern = tiled && 2 * nopat <= (unsigned long long)nnz &&
-                  ((uintptr_t)val.p | (uintptr_t)scol.p) % 16 == 0;
+                  ((uintptr_t)val.p | (uintptr_t)col.p | (uintptr_t)scol.p) % 16 == 0;
     }
     if (!pattern) {
         scol.reset();

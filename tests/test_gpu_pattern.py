@@ -98,3 +98,46 @@ def test_pattern_with_permuted_columns_and_special_values():
     rows = np.repeat(np.arange(A.nrows), A.row_lengths())
     hit = np.unique(rows[np.isin(A.col, [0, 20000])])
     assert np.array_equal(np.nonzero(~np.isfinite(y.cpu().numpy()))[0], hit)
+
+
+@pytest.mark.parametrize("sigma", [1, 256, 10 ** 9])
+@pytest.mark.parametrize("which", ["val", "col", "all"])
+def test_arrays_off_the_16_byte_grid_take_the_general_kernel(which, sigma):
+    """An allocator may return a pointer that is aligned for its values only:
+    the kernels that prefetch in 16-byte units are not used then."""
+    import torch
+    from paper_1307_6209_gb300 import sell
+    A = synth.dense(1000, 60)
+    x = torch.from_numpy(synth.block(A.ncols, 1, seed=4)[:, 0].copy()).cuda()
+    h = sell.sell_build(A, C=32, sigma=sigma)
+    want = torch.zeros(A.nrows, dtype=torch.float64, device="cuda")
+    sell.sell_spmv(h, x, want)
+    size = sell.sell_info(h).stored * (8 if which == "val" else 4)
+    h.free()
+    lib, shifted = sell.load(), []
+
+    def _alloc(nbytes, ctx, stream):
+        p = torch.cuda.caching_allocator_alloc(int(nbytes) + 16, torch.cuda.current_device(), stream or 0)
+        if which == "all" or nbytes == size:
+            p += 8
+            shifted.append(p)
+        return p
+
+    def _free(ptr, ctx, stream):
+        if ptr and ptr in shifted:
+            shifted.remove(ptr)
+            ptr -= 8
+        if ptr:
+            torch.cuda.caching_allocator_delete(ptr)
+
+    a, f = sell.ALLOC_FN(_alloc), sell.FREE_FN(_free)
+    assert lib.sell_set_allocator(a, f, None) == sell.SELL_OK
+    try:
+        h = sell.sell_build(A, C=32, sigma=sigma)
+        assert which == "all" or len(shifted) == 1
+        y = torch.zeros_like(want)
+        sell.sell_spmv(h, x, y)
+        assert torch.equal(y, want)
+        h.free()
+    finally:
+        assert lib.sell_set_allocator(sell.ALLOC_FN(), sell.FREE_FN(), None) == sell.SELL_OK
