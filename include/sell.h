@@ -214,6 +214,8 @@ SELL_API sell_status sell_spmv(sell_handle h, const void *x, void *y, uint32_t f
  * SELL_BUILD_PERMUTE_COLS).  The dot is summed in a fixed order over the
  * vector (1024 contiguous ranges, fixed trees), so its bits depend only on x
  * and y, not on the format, the launch or the run.  dot is a device pointer.
+ * Its scratch (8 KB) comes with the handle of a square matrix: the call
+ * allocates nothing and can be captured from the first one on.
  * Errors: those of sell_spmv, SELL_EINVAL (NULL dot, non-square A, HOST_IO). */
 SELL_API sell_status sell_spmv_dot(sell_handle h, const void *x, void *y, uint32_t flags, double *dot,
                                    void *stream);

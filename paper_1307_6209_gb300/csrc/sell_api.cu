@@ -134,7 +134,7 @@ void free_matrix(sell_matrix *h) {
     // every kernel that may still read the arrays must finish first
     (void)cudaDeviceSynchronize();
     void *ptrs[] = {h->val,    h->col,   h->cs,   h->cl,     h->srl,    h->perm,
-                    h->lchunk, h->lunit, h->cnt, h->cnt2, h->part, h->bsc, h->wsplit, h->dstat, h->dot_part,
+                    h->lchunk, h->lunit, h->cnt, h->cnt2, h->part, h->bsc, h->wsplit, h->dstat,
                     h->lrow,   h->lmeta, h->scol, h->sflag, h->lwork, h->lval, h->lcol, h->xpad, h->ppad};
     for (void *p : ptrs) h->al.put(p, nullptr);
     for (auto &sl : h->io) {
@@ -295,7 +295,6 @@ sell_status sell_spmv_dot(sell_handle h, const void *x, void *y, uint32_t flags,
     if (flags & (SELL_SPMV_HOST_IO | SELL_SPMV_HOST_DIRECT))
         return fail(SELL_EINVAL, "sell_spmv_dot: device vectors only");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    SELL_TRY(prepare_dot(h, s));
     SELL_TRY(sell_spmmv(h, x, 1, y, 1, 1, flags, stream));
     if (h->nrows == 0) {
         SELL_CUDA_TRY(cudaMemsetAsync(dot, 0, sizeof(double), s));

@@ -472,11 +472,12 @@ k_chunk_reduce(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, 
 
 // cs, and for the long chunks their index, first unit and first virtual warp
 // (and first packed one) in lpos/ubase/wbase; the totals go to cs[Nc] and *total.  tile: the tile sums.
+// dot_count (may be null): sell_spmv_dot's count of finished blocks, zero between products.
 __global__ void __launch_bounds__(kScanThreads)
 k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, int64_t Nc, int64_t per, int C,
               const ChunkSums *__restrict__ tile,
               int64_t *__restrict__ cs, int64_t *__restrict__ lpos, int64_t *__restrict__ ubase,
-              WorkBase *__restrict__ wbase, ChunkSums *__restrict__ total) {
+              WorkBase *__restrict__ wbase, ChunkSums *__restrict__ total, int64_t *__restrict__ dot_count) {
     __shared__ ChunkSums wt[32];
     __shared__ ChunkSums before;
     ChunkSums s = {0, 0, 0, 0, 0};
@@ -498,6 +499,7 @@ k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, i
             if (c == Nc - 1) {
                 cs[Nc] = v.stored;
                 *total = v;
+                if (dot_count) *dot_count = 0;
             }
         }
         __syncthreads();
@@ -1109,8 +1111,13 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
                                       permute_cols ? inv.as<int32_t>() : nullptr);
         SELL_CUDA_TRY(cudaGetLastError());
     }
-    // 5. chunk offsets, and the chunks that hold rows longer than kSeg
-    SELL_TRY(cs.alloc(al, (Nc + 1) * sizeof(int64_t), s));
+    // 5. chunk offsets, and the chunks that hold rows longer than kSeg.  The
+    // scratch of sell_spmv_dot follows the offsets of a square matrix, ready
+    // before the first product: allocated on first use, its clearing could be
+    // recorded in a graph instead of done.
+    const int64_t dot_words = N > 0 && N == A->ncols ? kDotRanges + 1 : 0;
+    SELL_TRY(cs.alloc(al, (Nc + 1 + dot_words) * sizeof(int64_t), s));
+    int64_t *dot_at = dot_words ? cs.as<int64_t>() + Nc + 1 : nullptr;
     DevBuf tile, lpos, ubase, wbase;
     ChunkSums total = {0, 0, 0, 0, 0};
     if (Nc > 0) {
@@ -1128,7 +1135,8 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_CUDA_TRY(cudaGetLastError());
         k_chunk_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(cl.as<int32_t>(), nlr, Nc, per, C, tp, cs.as<int64_t>(),
                                                             lpos.as<int64_t>(), ubase.as<int64_t>(),
-                                                            wbase.as<WorkBase>(), tp + nt);
+                                                            wbase.as<WorkBase>(), tp + nt,
+                                                            dot_at ? dot_at + kDotRanges : nullptr);
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_CUDA_TRY(cudaMemcpyAsync(&total, tp + nt, sizeof(total), cudaMemcpyDeviceToHost, s));
         SELL_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1263,6 +1271,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     h->val = val.release_ownership();
     h->col = (int32_t *)col.release_ownership();
     h->cs = (int64_t *)cs.release_ownership();
+    h->dot_part = reinterpret_cast<double *>(dot_at);
     h->cl = (int32_t *)cl.release_ownership();
     h->srl = (int32_t *)srl.release_ownership();
     h->perm = (int32_t *)perm.release_ownership();

@@ -23,7 +23,7 @@
 namespace sell {
 namespace {
 
-constexpr int kDotBlocks = 1024;
+constexpr int kDotBlocks = kDotRanges;
 constexpr int kDotThreads = 256;
 
 __device__ __forceinline__ double as_f64(double v) { return v; }
@@ -157,23 +157,6 @@ sell_status launch_dot(sell_matrix *h, const void *x, const void *y, double *out
                               ? run_dot(h, static_cast<const double *>(x), static_cast<const double *>(y), out, s)
                               : run_dot(h, static_cast<const float *>(x), static_cast<const float *>(y), out, s);
     if (e != cudaSuccess) return cuda_fail(e, "dot kernel launch");
-    return SELL_OK;
-}
-
-// The range sums and the count of finished blocks (allocated and cleared on
-// the first call, before the product is launched, so that the dot's launch
-// follows the product's directly).
-sell_status prepare_dot(sell_matrix *h, cudaStream_t s) {
-    if (h->dot_part || h->nrows == 0) return SELL_OK;
-    const size_t bytes = kDotBlocks * sizeof(double) + sizeof(double);
-    void *p = h->al.get(bytes, s);
-    if (!p) return fail(SELL_ENOMEM, "dot scratch allocation failed");
-    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, s);
-    if (e != cudaSuccess) {
-        h->al.put(p, s);
-        return cuda_fail(e, "clearing the dot scratch");
-    }
-    h->dot_part = static_cast<double *>(p);
     return SELL_OK;
 }
 

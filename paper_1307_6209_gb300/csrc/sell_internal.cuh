@@ -87,6 +87,9 @@ inline int rhs_block(int rem, int maxw) {
 // column at a time, in kernels of their own (sell_rowdot.cuh, WidePitch).
 constexpr int64_t kWidePitch = 1 << 28;
 
+// Ranges of sell_spmv_dot (sell_dot.cu).
+constexpr int kDotRanges = 1024;
+
 // A block of 3 or of 5 to 7 right-hand sides of binary32 vectors (7 of
 // binary64) runs as one of 4 or 8 on a copy of X with rows of that many
 // values: one vector load per gathered row and one pass over the matrix, where
@@ -162,7 +165,7 @@ struct sell_matrix {
     int32_t bulk_grid = 0, bulk_warps = 0, bulk_ring = 0;
     mutable uint32_t expire_us = 0;  // one-shot test hook of sell_test_expire_wait (0: off),
                                      // consumed by the next bulk-staged launch
-    double *dot_part = nullptr;  // range sums and block count of sell_spmv_dot (lazily allocated)
+    double *dot_part = nullptr;  // range sums and block count of sell_spmv_dot, behind cs (square matrices)
     // host-io staging (lazily allocated): kIoSlots slots used in turn, so that
     // the copies of one call overlap the kernels of the previous ones when
     // calls alternate streams.  A slot is reused only after its result has
@@ -224,7 +227,6 @@ cudaError_t launch_pad(const void *X, int64_t ldx, int64_t n, int cols, int K, s
 sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, sell_matrix *h);
 sell_status bulk_plan(sell_matrix *h, int64_t nwarps, cudaStream_t s);
 sell_status bulk_prepare(sell_matrix *h);
-sell_status prepare_dot(sell_matrix *h, cudaStream_t s);
 sell_status launch_dot(sell_matrix *h, const void *x, const void *y, double *out, cudaStream_t s);
 // scratch: per item, batch_item_scratch() bytes of device memory (or NULL for
 // items without long rows); NULL: the plan allocates its own.
