@@ -122,7 +122,10 @@ typedef struct {
 } sell_info_t;
 
 /* Device-memory callbacks: alloc(bytes, ctx, stream) returns a device pointer
- * or NULL; release(ptr, ctx, stream) frees it (may be called with NULL). */
+ * or NULL; release(ptr, ctx, stream) frees it (may be called with NULL).
+ * Pointers are aligned to 8 bytes at least.  (With 16 bytes, as every usual
+ * allocator gives, the column-pattern kernels and launch mode 2 are available;
+ * they look at the addresses of the arrays that they read in 16-byte units.) */
 typedef void *(*sell_alloc_fn)(size_t bytes, void *ctx, void *stream);
 typedef void (*sell_free_fn)(void *ptr, void *ctx, void *stream);
 

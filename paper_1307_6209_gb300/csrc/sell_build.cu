@@ -398,8 +398,7 @@ sell_status scan_exclusive(const T *in, int64_t n, int64_t *out, const Allocator
 // The sums over the chunks in one scan: chunk offsets (C * cl), long chunks
 // (cl > kSeg), their segments (ceil(cl / kSeg) each), the virtual warps of
 // sell_long.cuh and those of them with packed entries.  nlr[c] = rows of chunk c longer than kSeg.
-// The first long-row warp and pack of a chunk (8-byte aligned, as an allocator's
-// memory may be).
+// The first long-row warp and pack of a chunk.
 struct WorkBase {
     int64_t nwork, npack;
 };
@@ -552,7 +551,7 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
 // The long chunks (cl > kSeg), one warp per chunk: lchunk[i] = the i-th
 // long chunk; its ceil(cl / kSeg) work units are lunit[ubase + s] = {i, s};
 // lrow[i*C + k] = the lane of its k-th row longer than kSeg (lane order),
-// lmeta[i] = {m rows, mode, units of the chunk, 0}.  Mode 0: unit thread t
+// lmeta[i] = {m rows, mode, units of the chunk}.  Mode 0: unit thread t
 // takes lane t (its row's segment); mode 1, for chunks whose long rows are
 // few (8 m <= C): the chunk's unit threads take consecutive segments of one
 // long row after another, so a warp runs 32 segments of a long row instead of
@@ -563,7 +562,7 @@ __global__ void __launch_bounds__(256)
 k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, const int64_t *__restrict__ lpos,
              const int64_t *__restrict__ ubase, const WorkBase *__restrict__ wbase, const int64_t *__restrict__ cs, int64_t Nc, int64_t N, int C,
              int32_t *__restrict__ lchunk, int2 *__restrict__ lunit, int32_t *__restrict__ lrow,
-             int4 *__restrict__ lmeta, LongWork *__restrict__ lwork) {
+             LongMeta *__restrict__ lmeta, LongWork *__restrict__ lwork) {
     const int lane = threadIdx.x & 31;
     const int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int32_t width = c < Nc ? cl[c] : 0;
@@ -598,7 +597,7 @@ k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, co
     }
     if (lane == 0) {
         lchunk[i] = (int32_t)c;
-        lmeta[i] = make_int4(m, few ? 1 : 0, nseg, 0);
+        lmeta[i] = LongMeta{m, few ? 1 : 0, nseg};
     }
 }
 
@@ -1149,7 +1148,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_TRY(lchunk.alloc(al, nlong * sizeof(int32_t), s));
         SELL_TRY(lunit.alloc(al, nunits * sizeof(int2), s));
         SELL_TRY(lrow.alloc(al, (size_t)nlong * C * sizeof(int32_t), s));
-        SELL_TRY(lmeta.alloc(al, (size_t)nlong * sizeof(int4), s));
+        SELL_TRY(lmeta.alloc(al, (size_t)nlong * sizeof(LongMeta), s));
         if (total.nwork > 0) SELL_TRY(lwork.alloc(al, (size_t)total.nwork * sizeof(LongWork), s));
         if (total.npack > 0) {
             SELL_TRY(lval.alloc(al, (size_t)total.npack * kSeg * 32 * value_size(o->store_type), s));
@@ -1159,7 +1158,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
                                                                   lpos.as<int64_t>(), ubase.as<int64_t>(),
                                                                   wbase.as<WorkBase>(), cs.as<int64_t>(), Nc, N, C,
                                                                   lchunk.as<int32_t>(), lunit.as<int2>(),
-                                                                  lrow.as<int32_t>(), lmeta.as<int4>(),
+                                                                  lrow.as<int32_t>(), lmeta.as<LongMeta>(),
                                                                   lwork.as<LongWork>());
         SELL_CUDA_TRY(cudaGetLastError());
         SELL_TRY(cnt.alloc(al, nlong * C * sizeof(int32_t), s));
@@ -1264,7 +1263,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     h->lchunk = (int32_t *)lchunk.release_ownership();
     h->lunit = (int2 *)lunit.release_ownership();
     h->lrow = (int32_t *)lrow.release_ownership();
-    h->lmeta = (int4 *)lmeta.release_ownership();
+    h->lmeta = (LongMeta *)lmeta.release_ownership();
     h->cnt = (int32_t *)cnt.release_ownership();
     h->cnt2 = (int32_t *)cnt2.release_ownership();
     h->part = part.release_ownership();

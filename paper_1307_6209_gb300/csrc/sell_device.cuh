@@ -29,12 +29,20 @@ __host__ __device__ __forceinline__ int64_t offset_start(int64_t cs0, int32_t wi
 // whose first partial slot is u0 and which has nseg segments per row.
 // m < 0: segment i / (C / 32) of 32 neighbouring rows; else the 32 segments
 // from number 32 i of the chunk's m long rows, one row after another.  base:
-// where lane 0's first entry is.
-struct __align__(16) LongWork {
+// where lane 0's first entry is.  (8-byte aligned at most, here and below: an
+// allocator's memory need not be aligned for more.)
+struct LongWork {
     int32_t lc, c, nseg, m;
     int64_t base;
     int32_t i, u0;
 };
+
+// A long chunk's long rows, how its units take them (0: a unit thread per lane, 1: its
+// rows' segments one after another), and its segments per row.
+struct LongMeta {
+    int32_t m, mode, nseg;
+};
+static_assert(alignof(LongWork) <= 8 && alignof(LongMeta) <= 8, "an allocator's memory is 8-byte aligned");
 
 // --------------------------------------------------------- device helpers
 // Streaming loads for data touched once per product (val/col): do not allocate

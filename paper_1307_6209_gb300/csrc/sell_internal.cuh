@@ -143,7 +143,7 @@ struct sell_matrix {
     int64_t nlong = 0;
     int2 *lunit = nullptr;     // nunits long-row work units {long chunk, segment}
     int32_t *lrow = nullptr;   // nlong * C lanes of each long chunk's long rows
-    int4 *lmeta = nullptr;     // nlong {long rows, mode, units, 0} (sell_build.cu k_long_lists)
+    sell::LongMeta *lmeta = nullptr;  // nlong (sell_build.cu k_long_lists)
     int64_t nunits = 0;
     // long rows of single products (sell_long.cuh; null when C is no multiple of 32)
     sell::LongWork *lwork = nullptr;  // nlwork virtual warps

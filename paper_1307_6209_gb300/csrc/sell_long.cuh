@@ -51,7 +51,7 @@ struct LongArgs {
     const int64_t *cs;
     const int32_t *srl, *perm, *lchunk, *lrow;
     const int2 *lunit;
-    const int4 *lmeta;
+    const LongMeta *lmeta;
     const LongWork *lwork;
     const int32_t *lcol;
     Pattern pt;
@@ -109,19 +109,19 @@ __device__ __forceinline__ LongSeg unit_segment(const LongArgs &a, int64_t v) {
     const int t = (int)(v - u * a.C);
     if (u >= a.nwork) return LongSeg{};
     const int2 us = a.lunit[u];
-    const int4 meta = a.lmeta[us.x];
+    const LongMeta meta = a.lmeta[us.x];
     bool in = true;
     g.lc = us.x;
     g.u0 = u - us.y;
     g.c = a.lchunk[us.x];
-    if (meta.y == 0) {
+    if (meta.mode == 0) {
         g.l = t;
         g.s = us.y;
     } else {
         const int64_t i = (int64_t)us.y * a.C + t;  // beyond 32 bits for rows of more than 2^31 / C segments
-        const int64_t k = i / meta.z;
-        in = k < meta.x;
-        g.s = (int)(i - k * meta.z);
+        const int64_t k = i / meta.nseg;
+        in = k < meta.m;
+        g.s = (int)(i - k * meta.nseg);
         g.l = in ? a.lrow[(int64_t)us.x * a.C + k] : 0;
     }
     g.base = a.cs[g.c] + (int64_t)g.s * kSeg * a.C + g.l;

@@ -579,7 +579,7 @@ template <class VT, class XT, int K, int U, bool PIPE, class Acc>
 __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const int32_t *__restrict__ srl,
                                           const int32_t *__restrict__ perm, const int32_t *__restrict__ lchunk,
-                                          const int2 *__restrict__ lunit, const int4 *__restrict__ lmeta,
+                                          const int2 *__restrict__ lunit, const LongMeta *__restrict__ lmeta,
                                           const int32_t *__restrict__ lrow, Acc *part, int32_t *cnt,
                                           int32_t *cnt2, const XT *__restrict__ X, int64_t ldx, XT *Y,
                                           int64_t ldy, int64_t N, int C, int64_t v, int accumulate, int vec,
@@ -587,16 +587,16 @@ __device__ __forceinline__ void long_unit(const VT *__restrict__ val, const int3
     const int64_t u = v / C;
     const int t = (int)(v - u * C);
     const int2 us = lunit[u];
-    const int4 meta = lmeta[us.x];
+    const LongMeta meta = lmeta[us.x];
     int l, s;
-    if (meta.y == 0) {  // thread t takes lane t
+    if (meta.mode == 0) {  // thread t takes lane t
         l = t;
         s = us.y;
     } else {  // the chunk's threads take consecutive segments of each long row
         const int64_t i = (int64_t)us.y * C + t;  // beyond 32 bits for rows of more than 2^31 / C segments
-        const int64_t k = i / meta.z;
-        if (k >= meta.x) return;
-        s = (int)(i - k * meta.z);
+        const int64_t k = i / meta.nseg;
+        if (k >= meta.m) return;
+        s = (int)(i - k * meta.nseg);
         l = lrow[(int64_t)us.x * C + k];
     }
     const int64_t c = lchunk[us.x];

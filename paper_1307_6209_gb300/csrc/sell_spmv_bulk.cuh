@@ -132,7 +132,7 @@ struct Args {
     const int32_t *wsplit;   // nwarps + 1 chunk boundaries
     const int32_t *lchunk;
     const int2 *lunit;
-    const int4 *lmeta;
+    const LongMeta *lmeta;
     const int32_t *lrow;
     Acc *part;
     int32_t *cnt, *cnt2;
