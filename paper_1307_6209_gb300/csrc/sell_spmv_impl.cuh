@@ -37,15 +37,18 @@ namespace spmv_impl {
 
 // The rows of at most kSeg entries, one thread per row.  after_long: the long
 // rows' kernel (sell_long.cuh) runs ahead of this one, which ends only once
-// that has ended: the threads past the last row wait for it (launch_short
-// adds a block of them, so that there are some).
+// that has ended: the warps past the last row wait for it (launch_short adds a
+// block of them, so that there are some).  A warp with rows of its own does
+// not: they would be multiplied after the wait (unsorted lognormal rows
+// binary64 at one / eight vectors, 2000 rows 20.5 / 53 us then, 14.4 / 35 us
+// so; 50,000 rows 38 / 120 and 27 / 100 us).
 template <class VT, int K, int U, bool PIPE, class Acc, bool PAT, int CT, class LD>
 __device__ __forceinline__ void spmmv_body(SELL_SPMMV_PARAMS) {
     using XT = typename XType<VT>::T;
     dependents_may_start();  // a dot product's launch (sell_dot.cu)
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= N) {
-        if (after_long) wait_for_predecessor();
+        if (after_long && r - (threadIdx.x & 31) >= N) wait_for_predecessor();
         return;
     }
     short_row<VT, XT, K, U, PIPE, Acc, PAT, CT>(val, col, cs, srl, perm, pt, X, ldx, Y, ldy, C, (uint32_t)r, accumulate,
