@@ -144,53 +144,60 @@ __device__ __forceinline__ Dot2 shfl_acc(const Dot2 &v, int from) {
 }
 
 // Folds, for the lanes with `done`, `count` partials each (as fold_partials).
-// Many lanes at once (a chunk of rows of one length completes together) fold
-// their own; few are folded one by one with the whole warp's loads, 32
-// partials in one round trip instead of a few: a group of 256 takes one trip
-// to L2 instead of 16.  All 32 lanes call.
+// Either one row after another with the whole warp: lane t adds up column
+// t % K, 32 / K partials come with one load of all lanes, a few loads in
+// flight.  Or every row in its own lane, all rows at once.  A warp's binary64
+// addition takes 64 cycles of the FP64 pipe whatever its lanes do (about twice
+// that with the shuffle that brings its operand) and a round trip to L2 the
+// time of about kTrip of them, so what counts is the number of additions and
+// trips that follow each other.  Measured, before (rows one by one up to
+// four, K * n additions each) and after: a row of 10^4 entries in 10^4 short
+// ones, eight vectors, binary64 94 -> 45 us, binary32 72 -> 23 us; 1M unsorted
+// lognormal rows binary32 at eight vectors 288 -> 249 us; dense 1000^2 the
+// same (18.7 us; 21.9 with eight rows of 16 partials one by one).
+// All 32 lanes call.
+constexpr int kTrip = 10;
 template <int K, class PT>
 __device__ __forceinline__ void fold_warp(bool done, const PT *part, int64_t base, int64_t stride, int count, int C,
                                           int l, PT (&tot)[K]) {
     const int lane = threadIdx.x & 31;
     unsigned todo = __ballot_sync(0xffffffffu, done);
-    if (__popc(todo) > 4) {
+    const int rows = __popc(todo), most = __reduce_max_sync(0xffffffffu, done ? count : 0);
+    const int trips = 1 + (most - 1) / kFoldLoads<K> + (most - 1) % kFoldLoads<K>;  // fold_partials'
+    if (rows > 1 && rows * (kTrip + 2 * most) > kTrip * trips + K * most) {
         if (done) fold_partials<K, PT>(part, base, stride, count, C, l, tot);
         __syncwarp();
         return;
     }
     __syncwarp();  // the owner's fence holds for the loads of the other lanes
-    constexpr int Q = K == 1 ? 8 : 1;  // rounds of 32 loads in flight
+    constexpr int P = 32 / K, Q = K == 1 ? 8 : 4;  // partials per load, loads in flight (8 at K >= 2: 8 registers more)
+    const int e = lane % K;
     for (; todo; todo &= todo - 1) {
         const int owner = __ffs(todo) - 1;
         const int64_t b = __shfl_sync(0xffffffffu, base, owner);
         const int n = __shfl_sync(0xffffffffu, count, owner), ll = __shfl_sync(0xffffffffu, l, owner);
-        PT sum[K];
-        for (int i0 = 0; i0 < n; i0 += 32 * Q) {
-            PT p[Q][K];
+        PT sum;
+        for (int i0 = 0; i0 < n; i0 += P * Q) {
+            PT p[Q];
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
-                const int i = i0 + q * 32 + lane;
-                if (i < n) {
-#pragma unroll
-                    for (int e = 0; e < K; ++e) p[q][e] = PT::load_l2(part + ((b + i * stride) * C + ll) * K + e);
-                }
+                const int i = i0 + q * P + lane / K;
+                if (i < n) p[q] = PT::load_l2(part + ((b + i * stride) * C + ll) * K + e);
             }
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
-                const int m = min(32, n - i0 - q * 32);
+                const int m = min(P, n - i0 - q * P);
                 for (int t = 0; t < m; ++t) {
-#pragma unroll
-                    for (int e = 0; e < K; ++e) {
-                        const PT v = shfl_acc(p[q][e], t);
-                        if (i0 + q * 32 + t == 0) sum[e] = v;
-                        else sum[e].merge(v);
-                    }
+                    const PT v = shfl_acc(p[q], t * K + e);
+                    if (i0 + q * P + t == 0) sum = v;
+                    else sum.merge(v);
                 }
             }
         }
-        if (lane == owner) {
 #pragma unroll
-            for (int e = 0; e < K; ++e) tot[e] = sum[e];
+        for (int c = 0; c < K; ++c) {
+            const PT v = shfl_acc(sum, c);
+            if (lane == owner) tot[c] = v;
         }
     }
 }

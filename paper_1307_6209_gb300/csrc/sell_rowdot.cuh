@@ -537,13 +537,16 @@ __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ 
 }
 
 // Fold `count` partials of lane l, found at units base, base + stride, ...,
-// in that order (loads issued FB at a time, folds strictly in order).
+// in that order (kFoldLoads loads in flight; folds strictly in order).
+template <int K>
+constexpr int kFoldLoads = K >= 8 ? 2 : K >= 4 ? 4 : 16 / K;
+
 template <int K, class Acc>
 __device__ __forceinline__ void fold_partials(const Acc *part, int64_t base, int64_t stride, int count, int C,
                                               int l, Acc (&tot)[K]) {
 #pragma unroll
     for (int q = 0; q < K; ++q) tot[q] = Acc::load_l2(part + (base * C + l) * K + q);
-    constexpr int FB = K >= 8 ? 2 : (K >= 4 ? 4 : 16 / K);
+    constexpr int FB = kFoldLoads<K>;
     int i = 1;
     for (; i + FB <= count; i += FB) {
         Acc buf[FB][K];
