@@ -115,11 +115,13 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
         if (pat) kern = k_long<VT, K, U, P, AccL, true, Pitch>;
     }
     if constexpr (K == 4 && sizeof(VT) == 8) {
-        // with most of the entries the kernel has the chip to itself, and the
-        // loads in flight are worth the registers: dense 3000^2 94.8 us with
-        // unroll 2, 86 us so; 1M sorted lognormal rows, a third of the entries
-        // here, 113 and 115 us
-        if (2 * long_threads(h) * kSeg > h->nnz) kern = k_long<VT, K, 4, true, AccL, false, Pitch>;
+        // with most of the entries, in full segments, the kernel has the chip
+        // to itself, and the loads in flight are worth the registers: dense
+        // 3000^2 94 us with unroll 2, 86 us so.  1M sorted lognormal rows, a
+        // third of the entries here, 113 and 115 us; 60,000 in windows of 256,
+        // most lanes of whose virtual warps are idle, 39 and 46 us
+        const int64_t held = long_threads(h) * kSeg;  // entries of so many full segments
+        if (2 * held > h->nnz && 4 * held <= 5 * h->nnz) kern = k_long<VT, K, 4, true, AccL, false, Pitch>;
     }
     kern<<<blocks, kLongThreads, 0, s>>>(val, lval, a, part, cnt, cnt2, x, Pitch{(int32_t)(ldx * sizeof(XT))}, y, ldy,
                                          acc, vec);
