@@ -133,7 +133,7 @@ cudaError_t run_long(const sell_matrix *h, const void *X, int64_t ldx, void *Y, 
 // lengths (2M sorted lognormal rows binary64, unroll 4: block 128 132.7 us,
 // 256 137.4 us, 512 141.7 us; 64 gains nothing more).
 constexpr int kBlock = 128;
-constexpr int64_t kFewRows = 152 * 1024;  // half the chip's threads
+constexpr int64_t kFewRows = 152 * 2048;  // the chip's threads
 
 // One launch of a short-row kernel, behind the long rows' where there are any.
 template <class VT, class LD, class Kernel>
@@ -257,12 +257,19 @@ cudaError_t run_block(const sell_matrix *h, const void *X, int64_t ldx, void *Y,
                                         vec, s);
         }
         constexpr int U = K == 8 ? 2 : 4;
-        if constexpr (K == 2 && sizeof(VT) == 8) {
-            // few or even rows like the loads in flight better than the warps:
-            // 20,000 banded rows 6.8 us with unroll 4, 9.6 us with 2, 250,000
-            // 30.1 and 32.3 us, 100^3 stencil 94 and 96 us; 1M lognormal rows
-            // 74 and 70 us
-            if (h->nrows <= kFewRows || !h->nunits) return run<VT, K, 4, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
+        if constexpr (K > 1 && sizeof(VT) == 8) {
+            // Few rows like the loads in flight better than the warps, and so
+            // do even ones at two vectors.  Unroll 4 (2 at eight vectors)
+            // against half of it: two vectors, 280,000 lognormal rows sorted /
+            // in windows of 256 / unsorted 36 / 68 / 111 and 43 / 80 / 123 us,
+            // 1M sorted 72 and 70 us, 100^3 stencil 94 and 96 us; eight,
+            // 280,000 lognormal rows 76 / 220 / 387 and 84 / 235 / 406 us, 1M
+            // banded rows 408 and 401 us.  Four: 20,000 banded rows 12.3 and
+            // 15.8 us, but 500^2 Laplacian 18 and 14 us, 200,000 sorted
+            // lognormal rows 45 and 42 us.
+            const bool even = !h->nunits;
+            if (K == 4 ? even && h->nrows <= kFewRows / 8 : h->nrows <= kFewRows || (K == 2 && even))
+                return run<VT, K, U, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
         }
         return run<VT, K, sizeof(VT) == 8 ? U / 2 : U, true, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     }
