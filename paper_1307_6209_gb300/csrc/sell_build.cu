@@ -1220,6 +1220,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         // reads its columns).
         unsigned long long nopat = 0;
         for (unsigned long long n : end.nopat) nopat += n;
+        h->local = tiled && nnz > 0 && 4 * ((unsigned long long)nnz - nopat) >= (unsigned long long)nnz;
         // The kernel loads offsets and prefetches values and columns in 16-byte units.
         pattern = tiled && 2 * nopat <= (unsigned long long)nnz &&
                   ((uintptr_t)val.p | (uintptr_t)col.p | (uintptr_t)scol.p) % 16 == 0;

@@ -95,13 +95,11 @@ constexpr int kDotRanges = 1024;
 // values: one vector load per gathered row and one pass over the matrix, where
 // the blocks 2 + 1 or 4 + 2 + 1 take a load per value and a pass each.  The
 // kernels write the first `cols` columns, bits 4-7 of their vec argument (0:
-// all).  Worth a pass over X where a column has at least two entries on
-// average.  Measured at k = 3 / 5 / 7, binary32: 1M lognormal rows 192 / 244 /
+// all).  Worth it where pad_pays says so.  Measured at k = 3 / 5 / 7, binary32: 1M lognormal rows 192 / 244 /
 // 357 -> 105 / 129 / 139 us, 500,000 banded rows 50 / 80 / 116 -> 39 / 54 / 58
 // us, 100^3 stencil 92 / 127 / 182 -> 64 / 81 / 85 us.  Binary64 pays for the
 // columns that are not there with the FP64 pipe's time (100^3 stencil at k = 3
-// 160 -> 213 us, at 5 273 -> 380 us) except at 7: 393 -> 381 us, lognormal
-// 505 -> 352 us.
+// 160 -> 213 us, at 5 273 -> 380 us) except at 7: lognormal 505 -> 352 us.
 inline int pad_block(int rem, int maxw, bool f64) {
     if (rem == 3 && maxw >= 4 && !f64) return 4;
     return rem >= (f64 ? 7 : 5) && rem <= 7 && maxw >= 8 ? 8 : 0;
@@ -140,6 +138,7 @@ struct sell_matrix {
     // k_scatter_tiled): about stored / 32 offsets and one flag per 32 rows; null
     // unless most of the matrix lies in such slices
     int32_t *scol = nullptr, *sflag = nullptr;
+    bool local = false;        // at least a quarter of the entries in such slices: X is read from cache
     int64_t nlong = 0;
     int2 *lunit = nullptr;     // nunits long-row work units {long chunk, segment}
     int32_t *lrow = nullptr;   // nlong * C lanes of each long chunk's long rows
@@ -208,11 +207,25 @@ struct sell_batch {
 
 namespace sell {
 
-// Three columns trade one launch for another, which a small matrix of short
-// rows is not worth (20^3 stencil 14.4 -> 16.2 us; 5000 lognormal rows, with
-// long ones, 41 -> 21 us).
+// What a padded block costs is the copy of X, and what it saves are passes over
+// the matrix and loads of X, which are cheap where the columns come in patterns
+// (X lies in cache): there it takes 16 entries per column, 5 at seven vectors,
+// elsewhere 3 (2).  Binary64 at seven pays the FP64 pipe for the eighth column,
+// which patterns of more entries do not outweigh.  Measured in us, blocks /
+// padded, 1M rows binary32 at three, five and seven vectors: patterns of 3
+// entries 22 / 27, 23 / 37, 38 / 43; of 8 27 / 33, 31 / 43, 47 / 47; 100^3 stencil
+// 70 / 61, 93 / 76, 152 / 79; random columns, 2 per row 27 / 29, 37 / 39, 57 / 46;
+// 3 per row 37 / 33, 47 / 43, 72 / 51.  Binary64 at seven: patterns of 5 entries
+// 110 / 100, of 8 135 / 139, 100^3 stencil 360 / 386, but with long rows (dense
+// 1000^2) 58 / 45.  Three columns trade one launch for another, which a small
+// matrix of short rows is not worth (20^3 stencil 14.4 -> 16.2 us; 5000
+// lognormal rows, with long ones, 41 -> 21 us).
 inline bool pad_pays(const sell_matrix *h, int cols) {
-    return h->ncols > 0 && h->nnz >= 2 * h->ncols && (cols > 3 || h->nunits > 0 || h->nnz >= 500000);
+    const bool f64 = h->store_type == SELL_F64;
+    const int64_t least = h->local && !f64 ? (cols == 7 ? 5 : 16) : (cols == 7 ? 2 : 3);
+    if (h->ncols == 0 || h->nnz < least * h->ncols) return false;
+    if (h->local && f64 && !h->nunits && h->nnz >= 8 * h->ncols) return false;
+    return cols > 3 || h->nunits > 0 || h->nnz >= 500000;
 }
 
 // --------------------------------------------------------- launch entry points
