@@ -397,8 +397,8 @@ sell_status scan_exclusive(const T *in, int64_t n, int64_t *out, const Allocator
 
 // The sums over the chunks in one scan: chunk offsets (C * cl), long chunks
 // (cl > kSeg), their segments (ceil(cl / kSeg) each), the virtual warps of
-// sell_long.cuh and those of them with packed entries.  nlr[c] = rows of chunk c longer than kSeg.
-// The first long-row warp and pack of a chunk.
+// sell_long.cuh and the packed segments.  nlr[c] = rows of chunk c longer than kSeg.
+// The first long-row warp and packed segment of a chunk.
 struct WorkBase {
     int64_t nwork, npack;
 };
@@ -426,8 +426,7 @@ __device__ __forceinline__ ChunkSums sums_of(const int32_t *__restrict__ cl, con
     const int m = nlr[c];
     if (C % 32) return {(int64_t)C * w, 1, nseg, 0, 0};
     if (!few_long(m, C)) return {(int64_t)C * w, 1, nseg, nseg * (C / 32), 0};
-    const int64_t work = (m * nseg + 31) / 32;
-    return {(int64_t)C * w, 1, nseg, work, work};
+    return {(int64_t)C * w, 1, nseg, (m * nseg + 31) / 32, m * nseg};
 }
 __device__ __forceinline__ ChunkSums shfl_up(const ChunkSums &v, int o) {
     return {__shfl_up_sync(0xffffffffu, v.stored, o), __shfl_up_sync(0xffffffffu, v.nlong, o),
@@ -589,7 +588,7 @@ k_long_lists(const int32_t *__restrict__ cl, const int32_t *__restrict__ srl, co
             wk.nseg = nseg;
             wk.m = few ? m : -1;
             const int sl = (int)(k % (C / 32)), sg = (int)(k / (C / 32));
-            wk.base = few ? (wb.npack + k) * (kSeg * 32) : cs[c] + (int64_t)sg * kSeg * C + sl * 32;
+            wk.base = few ? (wb.npack + k * 32) * kSeg : cs[c] + (int64_t)sg * kSeg * C + sl * 32;
             wk.i = (int32_t)k;
             wk.u0 = (int32_t)u;
             lwork[wb.nwork + k] = wk;
@@ -801,6 +800,7 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
         const LongWork wk = lwork[w - npieces];
         if (wk.m < 0) return;
         const int64_t i = (int64_t)wk.i * 32 + lane, k = i / wk.nseg;
+        stride = (int)min((int64_t)32, (int64_t)wk.m * wk.nseg - i + lane);
         len = 0;
         if (k < wk.m) {
             const int64_t r = (int64_t)wk.c * C + lrow[(int64_t)wk.lc * C + k];
@@ -812,6 +812,10 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
         val = lval;
         col = lcol;
     }
+    // the row of the tile that this lane writes: the last one again where there
+    // are fewer than 32 (no branch around the writes: with one the build of 2M
+    // lognormal rows takes 107 us more)
+    const int row = min(lane, stride - 1);
     const int wmax = __reduce_max_sync(0xffffffffu, len);
     bool bad = false;
     auto mapped = [&](int32_t cidx) {
@@ -865,11 +869,11 @@ k_scatter_tiled(const int64_t *__restrict__ src_of, const int32_t *__restrict__ 
         }
         const int nj = min(kTileCols, j1 - jt);
         int32_t myoff = 0;
-        int64_t pos = at + (int64_t)(jt - j0) * stride + lane;
+        int64_t pos = at + (int64_t)(jt - j0) * stride + row;
         for (int q = 0; q < nj; ++q, pos += stride) {
             if (jt + q < wmax) {
-                const int32_t cc = tcol[warp][q][lane];
-                val[pos] = tval[warp][q][lane];
+                const int32_t cc = tcol[warp][q][row];
+                val[pos] = tval[warp][q][row];
                 col[pos] = cc;
                 const int32_t off = __shfl_sync(0xffffffffu, cc, lref) - fref;
                 same &= jt + q >= len || cc - first == off;
@@ -1153,8 +1157,8 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         SELL_TRY(lmeta.alloc(al, (size_t)nlong * sizeof(LongMeta), s));
         if (total.nwork > 0) SELL_TRY(lwork.alloc(al, (size_t)total.nwork * sizeof(LongWork), s));
         if (total.npack > 0) {
-            SELL_TRY(lval.alloc(al, (size_t)total.npack * kSeg * 32 * value_size(o->store_type), s));
-            SELL_TRY(lcol.alloc(al, (size_t)total.npack * kSeg * 32 * sizeof(int32_t), s));
+            SELL_TRY(lval.alloc(al, (size_t)total.npack * kSeg * value_size(o->store_type), s));
+            SELL_TRY(lcol.alloc(al, (size_t)total.npack * kSeg * sizeof(int32_t), s));
         }
         k_long_lists<<<(unsigned)((Nc + 7) / 8), 256, 0, s>>>(cl.as<int32_t>(), srl.as<int32_t>(),
                                                                   lpos.as<int64_t>(), ubase.as<int64_t>(),

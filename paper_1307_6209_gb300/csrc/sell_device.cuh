@@ -28,8 +28,8 @@ __host__ __device__ __forceinline__ int64_t offset_start(int64_t cs0, int32_t wi
 // A virtual warp of the long rows (sell_long.cuh): long chunk lc = chunk c,
 // whose first partial slot is u0 and which has nseg segments per row.
 // m < 0: segment i / (C / 32) of 32 neighbouring rows; else the 32 segments
-// from number 32 i of the chunk's m long rows, one row after another.  base:
-// where lane 0's first entry is.  (8-byte aligned at most, here and below: an
+// from number 32 i of the chunk's m long rows, one row after another (fewer in
+// the last).  base: where lane 0's first entry is.  (8-byte aligned at most, here and below: an
 // allocator's memory need not be aligned for more.)
 struct LongWork {
     int32_t lc, c, nseg, m;

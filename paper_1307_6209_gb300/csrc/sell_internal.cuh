@@ -148,7 +148,7 @@ struct sell_matrix {
     sell::LongWork *lwork = nullptr;  // nlwork virtual warps
     int64_t nlwork = 0;
     void *lval = nullptr;      // entries of the virtual warps of chunks with few long rows,
-    int32_t *lcol = nullptr;   //   nlpack * kSeg * 32 of each
+    int32_t *lcol = nullptr;   //   kSeg of each per segment
     int32_t *cnt = nullptr;    // nlong * C per-row segment counters (zero at rest)
     int32_t *cnt2 = nullptr;   // nunits * C group counters of very long rows (zero at rest)
     void *part = nullptr;      // segment partials: nunits * C * part_k * 8 bytes

@@ -8,8 +8,9 @@
 // long row after another -- only as many virtual warps as there are segments.
 // The chunk holds such a row with a stride of C entries, one useful entry per
 // 32-byte sector; its virtual warps therefore have a copy of their entries,
-// entry j of lane t at base + j * 32 + t (lval, lcol: at most an eighth of the
-// chunk they come from), so that they read like a chunk of 32 full rows.
+// entry j of lane t at base + j * n + t, n the lanes that have a segment (lval,
+// lcol: kSeg entries per segment, less than a quarter of the chunk they come
+// from), so that they read like a chunk of n full rows.
 // Chunk heights that are not a multiple of 32 go through the units of
 // sell_rowdot.cuh instead (lwork is null).
 //
@@ -95,7 +96,7 @@ __device__ __forceinline__ LongSeg long_segment(const LongArgs &a, int64_t w, in
         in = k < wk.m;
         g.s = (int)(i - k * wk.nseg);
         g.l = in ? a.lrow[(int64_t)wk.lc * a.C + k] : 0;
-        g.stride = 32;
+        g.stride = (int)min((int64_t)32, (int64_t)wk.m * wk.nseg - (int64_t)wk.i * 32);
     }
     g.packed = wk.m >= 0;
     finish_segment(a, g, in);
