@@ -118,7 +118,10 @@ typedef struct {
     int32_t has_perm;     /* 0 when sigma <= 1 (the permutation is identity) */
     double beta;          /* Eq. "beta": nnz / stored (1 when stored = 0) */
     double zeta;          /* Eq. "cv": coefficient of variation of row lengths */
-    size_t device_bytes;  /* device memory owned by the handle */
+    size_t device_bytes;  /* device memory owned by the handle: the format and the scratch of one
+                             right-hand side, and from their first use on the padded copy of X (8
+                             values per column) and its scratch (64 bytes per segment and row of the
+                             chunks with long rows), whichever of the padded widths was used */
 } sell_info_t;
 
 /* Device-memory callbacks: alloc(bytes, ctx, stream) returns a device pointer

@@ -369,6 +369,7 @@ sell_status sell_info(sell_handle h, sell_info_t *info) {
     info->has_perm = h->perm != nullptr;
     info->beta = h->beta;
     info->zeta = h->zeta;
+    std::lock_guard<std::mutex> lock(h->pad_mu);
     info->device_bytes = h->device_bytes;
     return SELL_OK;
 }

@@ -155,7 +155,7 @@ struct sell_matrix {
     int32_t part_k = 0;
     void *xpad = nullptr;      // padded copy of X (pad_block): ncols * 8 values, allocated on first use
     void *ppad = nullptr;      // segment partials of padded blocks: nunits * C * 8 * 8 bytes, allocated with xpad
-    std::mutex pad_mu;         // held from the copy's launch to its product's
+    std::mutex pad_mu;         // held from the copy's launch to its product's, and for device_bytes
     // bulk-staged SpMV (launch mode 2), prepared by sell_set_launch
     int32_t *bsc = nullptr;    // nchunks staged columns per chunk
     int32_t *wsplit = nullptr; // wsplit_n + 1 per-warp chunk boundaries

@@ -68,9 +68,12 @@ bool make_pad(sell_matrix *h, cudaStream_t s) {
         return false;
     }
     if (st != cudaStreamCaptureStatusNone) return false;
-    if (part && !(h->ppad = h->al.get((size_t)h->nunits * h->C * 8 * 8, s))) return false;
-    if (!h->xpad) h->xpad = h->al.get((size_t)h->ncols * 8 * (h->store_type == SELL_F64 ? 8 : 4), s);
-    return h->xpad != nullptr;
+    auto take = [&](void *&p, size_t bytes) {
+        if (!p && (p = h->al.get(bytes, s))) h->device_bytes += bytes;
+        return p != nullptr;
+    };
+    if (part && !take(h->ppad, (size_t)h->nunits * h->C * 8 * 8)) return false;
+    return take(h->xpad, (size_t)h->ncols * 8 * (h->store_type == SELL_F64 ? 8 : 4));
 }
 
 }  // namespace
