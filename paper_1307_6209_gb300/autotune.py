@@ -6,7 +6,10 @@ work (Sec. 6) and notes that the best sigma is matrix dependent (Sec. 3.4,
 Sec. 5.3).  Stage 1 builds every (C, sigma) candidate and times the SpMV with
 the default launch; stage 2 sweeps (block, unroll, pipeline) on the best
 formats (software pipelining at every number of right-hand sides, bulk
-staging for single right-hand sides, where they exist).  All
+staging for single right-hand sides, where they exist).  The library's own
+launch is among the candidates: at one right-hand side the sweep's block 128
+with pipelining is the same kernel, at more, where the blocks of columns have
+launches of their own, it is timed as (0, 0, -1).  All
 timing goes through the C ABI (CUDA events on the given stream).  Results are
 cached in a JSON file keyed by a matrix signature (sizes, longest row, the
 coefficient of variation of Eq. "cv", storage type, right-hand sides).
@@ -127,20 +130,18 @@ def tune(A, store_type: int = sell.SELL_F64, k: int = 1, Cs=(32, 64, 128), sigma
     best = None
     for r in formats[:keep]:
         h = built[(r["C"], r["sigma"])]
-        for b in blocks:
-            for u in unrolls:
-                for p in pipelines:
-                    if (p == 1 and k > 2) or (p == 2 and k > 1):
-                        continue  # modes 1 and 2 exist for k <= 2 and k = 1
-                    try:
-                        sell.sell_set_launch(h, b, u, p)
-                    except sell.SellError:
-                        continue  # e.g. mode 2 with a C it does not take
-                    us = _time(lambda: product(h), stream, reps)
-                    launches.append({"C": r["C"], "sigma": r["sigma"], "block": b, "unroll": u, "pipeline": p,
-                                     "us": us})
-                    if best is None or us < best.us:
-                        best = Choice(r["C"], r["sigma"], b, u, us, flops / us / 1e3, p)
+        own = [(0, 0, -1)] if k > 1 else []  # before anything is set
+        for b, u, p in own + [(b, u, p) for b in blocks for u in unrolls for p in pipelines]:
+            if p == 2 and k > 1:
+                continue  # the bulk-staged kernel takes one right-hand side
+            try:
+                sell.sell_set_launch(h, b, u, p)
+            except sell.SellError:
+                continue  # e.g. mode 2 with a C it does not take
+            us = _time(lambda: product(h), stream, reps)
+            launches.append({"C": r["C"], "sigma": r["sigma"], "block": b, "unroll": u, "pipeline": p, "us": us})
+            if best is None or us < best.us:
+                best = Choice(r["C"], r["sigma"], b, u, us, flops / us / 1e3, p)
     for h in built.values():
         h.free()
     if cache:

@@ -217,6 +217,11 @@ cudaError_t pick_u(const sell_matrix *h, const void *X, int64_t ldx, void *Y, in
         if (u >= 2) return run<VT, K, 2, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
         return run<VT, K, 1, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
     } else {
+        if constexpr (K == 1 && PIPE) {
+            constexpr int own = sizeof(VT) == 8 ? 2 : 4;  // the library's choice and its kernel (run_block)
+            if (h->C == 32 && u == own)
+                return launch_short<VT>(k_spmv_short<VT, own, true, Acc, 32>, h, X, ldx, Y, ldy, acc, vec, s);
+        }
         if (u >= 8) return run<VT, K, 8, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
         if (u >= 4) return run<VT, K, 4, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
         if (u >= 2) return run<VT, K, 2, PIPE, Acc>(h, X, ldx, Y, ldy, acc, vec, s);
