@@ -299,8 +299,8 @@ __device__ __forceinline__ void long_rows(const VT *__restrict__ val, const VT *
             if (!g.packed && a.pt.flag[g.r >> 5]) {
                 const int64_t cs0 = a.cs[g.c];
                 const int32_t *op = a.pt.off + offset_start(cs0, a.pt.cl[g.c], g.l >> 5, g.r >> 5) + g.s * kSeg;
-                chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, vp, op, __ldg(a.col + cs0 + g.l), g.stride, 0, n, X,
-                                                          ldx, vec, pol);
+                chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, vp, op, __ldg(a.col + cs0 + g.l), g.stride, n, X, ldx,
+                                                          vec, pol);
                 done = true;
             }
         }

@@ -4,10 +4,11 @@
 // loop that runs under a fixed memory budget, code that runs inside another
 // framework's memory pool, or a latency-critical path where an allocation
 // (and the synchronisation it may imply) is not acceptable.  sell_spmmv can
-// allocate in two cases -- host-buffer staging, and a larger long-row scratch
-// the first time more right-hand sides are used -- so this entry point
-// computes the same product with its long-row scratch in one fixed device
-// array that the library holds for the whole process.
+// allocate in three cases -- host-buffer staging, a larger long-row scratch the
+// first time more right-hand sides are used, and a padded copy of X the first
+// time they are 3 or 5 to 7 -- so this entry point computes the same product
+// with its long-row scratch in one fixed device array that the library holds
+// for the whole process.
 //
 // The array has kScratchBytes bytes on every device that loads the library.
 // In host code `g_noalloc_scratch` names a host-side stand-in, not the device

@@ -405,19 +405,17 @@ __device__ __forceinline__ void chain(Acc (&acc)[K], const VT *__restrict__ vp,
 
 // The same chain for a row of a slice with one column pattern: entry j lies
 // in column first + op[j], op the same for the whole warp (16-byte loads that
-// all lanes share).  U is 2 or a multiple of 4, j0 a multiple of U; CT is the chunk height
-// where it is known at compile time (the strides become constants of the
-// load instructions), else 0.
+// all lanes share).  U is 2 or a multiple of 4; CT is the chunk height where it
+// is known at compile time (the strides become constants of the load
+// instructions), else 0.
 template <class VT, class XT, int K, int U, bool PIPE, int CT, class Acc>
 __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restrict__ vp,
-                                              const int32_t *__restrict__ op, int32_t first, int C, int j0, int j1,
+                                              const int32_t *__restrict__ op, int32_t first, int C, int j1,
                                               const XT *__restrict__ X, Pitch ldx, int vec, uint64_t pol) {
     const int stride = CT ? CT : C;
     const XT *xp = x_row(X, ldx, first);
-    op += j0;
-    vp += (int64_t)j0 * stride;
     constexpr int XB = K >= 8 && U > 2 ? 2 : U;  // rows of X in flight
-    int j = j0;
+    int j = 0;
     auto group = [&](const VT (&v)[U], const int32_t (&o)[U], int n) {
 #pragma unroll
         for (int b = 0; b < U; b += XB) {
@@ -499,23 +497,21 @@ __device__ __forceinline__ void chain_pattern(Acc (&acc)[K], const VT *__restric
     }
 }
 
-// The chain over entries j0..j1-1 of sorted row r = lane l of chunk c.
+// The chain over the n entries of sorted row r = lane l of chunk c.
 // PAT: the matrix has slices with one column pattern.
 template <class VT, class XT, int K, int U, bool PIPE, class Acc, bool PAT, int CT, class LD>
 __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ val, const int32_t *__restrict__ col,
                                           const int64_t *__restrict__ cs, const Pattern &pt, int C, int64_t r,
-                                          int64_t c, int l, int j0, int j1, const XT *__restrict__ X, LD ldx,
-                                          int vec, uint64_t pol) {
+                                          int64_t c, int l, int n, const XT *__restrict__ X, LD ldx, int vec,
+                                          uint64_t pol) {
     const int64_t cs0 = cs[c];
     const int64_t base = cs0 + l;
     if constexpr (PAT) {
         // one request brings the warp's values to L2 (the first lane's row
         // stands for all), so that the loads below wait for L2 and not for HBM
-        constexpr bool PREFETCH = sizeof(XT) == 4 || K < 4;  // wider binary64 products are bound by the FP64 pipe
         const int32_t width = pt.cl[c];
-        const int n = j1 - j0;
-        const int64_t at = cs0 + (int64_t)j0 * C + (int64_t)(l & ~31) * n;
-        const bool ask = PREFETCH && (l & 31) == 0 && n > 0;
+        const int64_t at = cs0 + (int64_t)(l & ~31) * n;
+        const bool ask = (l & 31) == 0 && n > 0;
         const int32_t flag = pt.flag[r >> 5];
         prefetch_l2(ask, val + at, (uint32_t)(n * 32 * sizeof(VT)), pol);
         if (flag) {
@@ -524,16 +520,16 @@ __device__ __forceinline__ void row_chain(Acc (&acc)[K], const VT *__restrict__ 
             const int32_t *op = pt.off + offset_start(cs0, width, l >> 5, r >> 5);
             if constexpr (sizeof(XT) == 4) {  // binary64 waits for the FP64 pipe, not for its addresses
                 if (C == 32) {
-                    chain_pattern<VT, XT, K, U, PIPE, 32, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+                    chain_pattern<VT, XT, K, U, PIPE, 32, Acc>(acc, val + base, op, first, C, n, X, ldx, vec, pol);
                     return;
                 }
             }
-            chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, j0, j1, X, ldx, vec, pol);
+            chain_pattern<VT, XT, K, U, PIPE, 0, Acc>(acc, val + base, op, first, C, n, X, ldx, vec, pol);
             return;
         }
         prefetch_l2(ask, col + at, (uint32_t)(n * 128), pol);
     }
-    chain<VT, XT, K, U, PIPE, Acc, CT>(acc, val + base, col + base, C, j0, j1, X, ldx, vec, pol);
+    chain<VT, XT, K, U, PIPE, Acc, CT>(acc, val + base, col + base, C, 0, n, X, ldx, vec, pol);
 }
 
 // Fold `count` partials of lane l, found at units base, base + stride, ...,
@@ -565,8 +561,8 @@ __device__ __forceinline__ void fold_partials(const Acc *part, int64_t base, int
     }
 }
 
-// One thread of a long-row work unit (batches and the bulk-staged kernel; the
-// single products' long rows are in sell_long.cuh).  Units are (long chunk lc, segment s)
+// One thread of a long-row work unit (the bulk-staged kernel's; those of the
+// other products and of batches are in sell_long.cuh).  Units are (long chunk lc, segment s)
 // pairs, numbered chunk by chunk (lunit[u] = {lc, s}); a unit has C threads,
 // virtual thread v = u*C + l takes lane l.  part holds K Accs per (unit,
 // lane); cnt one counter per (long chunk, lane) and cnt2 one per (unit,
@@ -673,7 +669,7 @@ __device__ __forceinline__ void short_row(const VT *__restrict__ val, const int3
 #pragma unroll
         for (int q = 0; q < K; ++q) acc[q].init(XT(0));
     }
-    row_chain<VT, XT, K, U, PIPE, Acc, PAT, CT>(acc, val, col, cs, pt, C, r, c, l, 0, L, X, ldx, vec, pol);
+    row_chain<VT, XT, K, U, PIPE, Acc, PAT, CT>(acc, val, col, cs, pt, C, r, c, l, L, X, ldx, vec, pol);
     XT yo[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) yo[q] = acc[q].result();
