@@ -48,6 +48,7 @@ struct BuildStats {
     int max_rl;
     unsigned long long sumsq;
     unsigned long long nopat[kNopatSlots];  // entries in slices without a column pattern
+    unsigned int far;  // slices whose rows begin far apart, of those looked at (k_chunk_len)
 };
 enum : unsigned int {
     kErrRpt0 = 1u,
@@ -510,10 +511,15 @@ k_chunk_apply(const int32_t *__restrict__ cl, const int32_t *__restrict__ nlr, i
 // srl, cl, and src[r] = where sorted row r's entries begin in the CRS arrays:
 // the scatter then waits for one load instead of a chain of three (length,
 // perm, rpt) before a row's entries.
+// Every near_step-th slice (32 sorted rows; 0: none) also says whether its rows
+// begin kNear columns or more apart (st->far).
+constexpr int kNear = 4096;        // rows of X of up to 32 bytes that L1 holds
+constexpr int kNearSlices = 1024;  // slices looked at, about
 __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__restrict__ perm,
                             const int64_t *__restrict__ rpt, int64_t N, int64_t Np, int C, int32_t *__restrict__ srl,
                             int64_t *__restrict__ src, int32_t *__restrict__ cl, int32_t *__restrict__ nlr,
-                            int32_t *__restrict__ inv) {
+                            int32_t *__restrict__ inv, const int32_t *__restrict__ col_in, int64_t near_step,
+                            BuildStats *st) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool warp_chunks = (C % 32) == 0;
     // the loop trip count is uniform across a warp because Np is a multiple of
@@ -530,6 +536,12 @@ __global__ void k_chunk_len(const int32_t *__restrict__ rl, const int32_t *__res
         if (live) {
             srl[r] = len;
             if (r < N) src[r] = rpt[perm ? perm[r] : r];
+        }
+        if (near_step && (r >> 5) % near_step == 0) {
+            const int32_t first = len > 0 ? col_in[src[r]] : 0;
+            const int32_t lo = __reduce_min_sync(0xffffffffu, len > 0 ? first : 0x7FFFFFFF);
+            const int32_t hi = __reduce_max_sync(0xffffffffu, len > 0 ? first : 0);
+            if ((threadIdx.x & 31) == 0 && (int64_t)hi - lo >= kNear) atomicAdd(&st->far, 1u);
         }
         if (warp_chunks) {
             int32_t m = len;
@@ -1109,11 +1121,14 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
     }
     const bool permute_cols = (o->flags & SELL_BUILD_PERMUTE_COLS) != 0;
     if (permute_cols && N > 0) SELL_TRY(inv.alloc(al, N * sizeof(int32_t), s));
+    // (for the padded blocks of binary32 vectors, sell_internal.cuh)
+    const int64_t near_step = C % 32 == 0 && nnz > 0 && o->store_type != SELL_F64 ? std::max<int64_t>(1, Np / 32 / kNearSlices) : 0;
     if (Np > 0) {
         int g = grid_for(Np, 256);
         k_chunk_len<<<g, 256, 0, s>>>(rl.as<int32_t>(), sorted ? perm.as<int32_t>() : nullptr, rpt, N, Np,
                                       C, srl.as<int32_t>(), src.as<int64_t>(), cl.as<int32_t>(), cl.as<int32_t>() + Nc,
-                                      permute_cols ? inv.as<int32_t>() : nullptr);
+                                      permute_cols ? inv.as<int32_t>() : nullptr, col_in, near_step,
+                                      stats.as<BuildStats>());
         SELL_CUDA_TRY(cudaGetLastError());
     }
     // 5. chunk offsets, and the chunks that hold rows longer than kSeg.  The
@@ -1224,6 +1239,7 @@ sell_status build_format(const sell_csr *A, const sell_opts *o, cudaStream_t s, 
         // reads its columns).
         unsigned long long nopat = 0;
         for (unsigned long long n : end.nopat) nopat += n;
+        h->near = near_step > 0 && 2 * (int64_t)end.far * near_step <= Np / 32;
         h->local = tiled && nnz > 0 && 4 * ((unsigned long long)nnz - nopat) >= (unsigned long long)nnz;
         // The kernel loads offsets and prefetches values and columns in 16-byte units.
         pattern = tiled && 2 * nopat <= (unsigned long long)nnz &&

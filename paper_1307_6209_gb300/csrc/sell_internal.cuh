@@ -138,7 +138,8 @@ struct sell_matrix {
     // k_scatter_tiled): about stored / 32 offsets and one flag per 32 rows; null
     // unless most of the matrix lies in such slices
     int32_t *scol = nullptr, *sflag = nullptr;
-    bool local = false;        // at least a quarter of the entries in such slices: X is read from cache
+    bool local = false;        // at least a quarter of the entries in such slices
+    bool near = false;         // most slices' rows begin close together: X is read from cache (not binary64)
     int64_t nlong = 0;
     int2 *lunit = nullptr;     // nunits long-row work units {long chunk, segment}
     int32_t *lrow = nullptr;   // nlong * C lanes of each long chunk's long rows
@@ -208,12 +209,14 @@ struct sell_batch {
 namespace sell {
 
 // What a padded block costs is the copy of X, and what it saves are passes over
-// the matrix and loads of X, which are cheap where the columns come in patterns
-// (X lies in cache): there it takes 16 entries per column, 5 at seven vectors,
-// elsewhere 3 (2).  Binary64 at seven pays the FP64 pipe for the eighth column,
-// which patterns of more entries do not outweigh.  Measured in us, blocks /
+// the matrix and loads of X, which are cheap where neighbouring rows' columns lie
+// close together (X lies in cache): there it takes 16 entries per column, 5 at
+// seven vectors, elsewhere, and with long rows, which make every pass two
+// launches, 3 (2).  Binary64 at seven pays the FP64 pipe for the
+// eighth column, which patterns of more entries do not outweigh.  Measured in us, blocks /
 // padded, 1M rows binary32 at three, five and seven vectors: patterns of 3
-// entries 22 / 27, 23 / 37, 38 / 43; of 8 27 / 33, 31 / 43, 47 / 47; 100^3 stencil
+// entries 22 / 27, 23 / 37, 38 / 43; of 8 27 / 33, 31 / 43, 47 / 47; bands without a
+// pattern of 5 28 / 37, 37 / 43, 54 / 46; 100^3 stencil
 // 70 / 61, 93 / 76, 152 / 79; random columns, 2 per row 27 / 29, 37 / 39, 57 / 46;
 // 3 per row 37 / 33, 47 / 43, 72 / 51.  Binary64 at seven: patterns of 5 entries
 // 110 / 100, of 8 135 / 139, 100^3 stencil 360 / 386, but with long rows (dense
@@ -222,7 +225,7 @@ namespace sell {
 // lognormal rows, with long ones, 41 -> 21 us).
 inline bool pad_pays(const sell_matrix *h, int cols) {
     const bool f64 = h->store_type == SELL_F64;
-    const int64_t least = h->local && !f64 ? (cols == 7 ? 5 : 16) : (cols == 7 ? 2 : 3);
+    const int64_t least = h->near && !h->nunits && !f64 ? (cols == 7 ? 5 : 16) : (cols == 7 ? 2 : 3);
     if (h->ncols == 0 || h->nnz < least * h->ncols) return false;
     if (h->local && f64 && !h->nunits && h->nnz >= 8 * h->ncols) return false;
     return cols > 3 || h->nunits > 0 || h->nnz >= 500000;
